@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "eloc.cuh"
 #include "metro.cuh"
 #include "prop.cuh"
 #include "tc.cuh"
@@ -115,6 +116,23 @@ extern "C" int64_t gna_num_params(const gna_model_desc* d) {
 
 namespace gna {
 
+// Tensor-core local energy: split operands on the warp-tiled kernel where the balls fit its
+// shared memory, else (and in BF16) on the tensor-memory kernel.
+static gna_status tensor_eloc_workspace(const gna_graph* g, const Dims& m, int64_t B, size_t* bytes, int split) {
+  if (split) {
+    gna_status st = el_workspace(g, m, B, bytes);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
+  return tc_workspace(g, m, TC_ELOC, B, bytes, split);
+}
+static gna_status tensor_eloc_run(const TcCall& c, void* ws, size_t ws_bytes, cudaStream_t stream) {
+  if (c.split) {
+    gna_status st = el_run(c, ws, ws_bytes, stream);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
+  return tc_run(c, ws, ws_bytes, stream);
+}
+
 static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int op, int64_t B, size_t* bytes) {
   const Dims m = make_dims(g, d);
   const int sp = simt_prec(d);
@@ -125,11 +143,11 @@ static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int 
     case GNA_OP_LOCAL_ENERGY_FULL:
       return simt_workspace(g, m, sp, 1, B, bytes);
     case GNA_OP_LOCAL_ENERGY_INCREMENTAL:
-      if (tensor_prec(d)) return tc_workspace(g, m, TC_ELOC, B, bytes, split_prec(d));
+      if (tensor_prec(d)) return tensor_eloc_workspace(g, m, B, bytes, split_prec(d));
       return simt_workspace(g, m, sp, 2, B, bytes);
     case GNA_OP_LOCAL_ENERGY_LOGPSI: {
       // the local-energy call (its own forward gives log Psi), or the two calls in turn
-      if (tensor_prec(d)) return tc_workspace(g, m, TC_ELOC, B, bytes, split_prec(d));
+      if (tensor_prec(d)) return tensor_eloc_workspace(g, m, B, bytes, split_prec(d));
       size_t a = 0, b = 0;
       gna_status st = simt_workspace(g, m, sp, 0, B, &a);
       if (st != GNA_OK) return st;
@@ -245,7 +263,7 @@ extern "C" gna_status gna_local_energy(const gna_graph* g, const gna_model_desc*
   const Dims m = make_dims(g, d);
   if (tensor_prec(d) && mode == GNA_ELOC_INCREMENTAL) {
     TcCall tc{g, m, TC_ELOC, (const float*)theta, spins, B, nullptr, eloc, dlogpsi_bonds, split_prec(d)};
-    return tc_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
+    return tensor_eloc_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
   }
   SimtCall sc{};
   sc.g = g;
@@ -271,7 +289,7 @@ extern "C" gna_status gna_local_energy_logpsi(const gna_graph* g, const gna_mode
   if (st != GNA_OK) return st;
   if (tensor_prec(d)) {
     TcCall tc{g, make_dims(g, d), TC_ELOC, (const float*)theta, spins, B, logpsi, eloc, nullptr, split_prec(d)};
-    return tc_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
+    return tensor_eloc_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
   }
   st = gna_forward(g, d, theta, spins, B, logpsi, workspace, workspace_bytes, stream);
   if (st != GNA_OK) return st;

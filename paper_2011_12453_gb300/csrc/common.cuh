@@ -41,6 +41,13 @@ struct DevGraph {
   const int* row_pack = nullptr;       // [sum]  v | (start of the row's entries within the bond's << 16)
   const int16_t* nbr_pos16 = nullptr;  // [...]  nbr_pos, 32767 outside ball_Lmax
   const int* bond_ent = nullptr;       // [E]    start of bond e's entries in nbr_pos / nbr_pos16
+  // The same rows for the warp-tiled kernels: neighbour positions two at a time, every bond's
+  // part on a 16-byte boundary (asynchronous 16-byte copies).
+  const int* rec = nullptr;         // [sum][2]  v | (pairs of the row << 16), first pair within the bond's
+  const uint32_t* pairs = nullptr;  // [...]     two 16-bit positions p as 4 p + (p & 1), 0xFFFF outside ball_Lmax
+  // [E][32] bond e: first row in rec (even), first pair (a multiple of 4), J (2 ints), i, j, 0, 0,
+  // |ball_0| .. |ball_8| at 8 .. 16 -- the pairs of the first |ball_l| rows follow at 16 + l, l >= 1
+  const int* bond_info = nullptr;
 };
 
 // Diagonal element of bond e's Hamiltonian for S^z eigenvalues s_i/2, s_j/2 (float64):
@@ -59,7 +66,8 @@ struct gna_graph {
   std::vector<double> h_J;  // off-diagonal couplings
   std::vector<int> max_ball;  // [Lmax+1] max over bonds of |ball_l|
   std::vector<int> max_span;  // [Lmax+1] max over bonds of sum of degrees over ball_l rows
-  int max_deg = 0;
+  std::vector<int> max_pairs; // [Lmax+1] max over bonds of the neighbour pairs of ball_l's rows
+  int max_deg = 0, min_deg = 0;
   bool pack_ok = true;  // every bond's entries fit the 16-bit starts of row_pack
   std::vector<void*> allocations;
 };

@@ -5,7 +5,6 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
-#include <set>
 #include <utility>
 #include <vector>
 
@@ -23,6 +22,8 @@ struct HostGraph {
   std::vector<int> ball_off, ball_size, ball_vert, row_nbr, nbr_pos, max_ball, max_span;
   std::vector<int> ball_span, row_pack, bond_ent;  // compact forms, see DevGraph
   std::vector<int16_t> nbr_pos16;
+  std::vector<int> rec, bond_info, max_pairs;  // rows with neighbour pairs, see DevGraph
+  std::vector<uint32_t> pairs;
   bool pack_ok = true;
 };
 
@@ -33,14 +34,15 @@ gna_status validate(int32_t n_sites, int32_t n_edges, const int32_t* edges, cons
   if (max_layers < 0 || max_layers > kMaxL) return GNA_ERR_INVALID_ARG;
   if (n_edges > 0 && edges == nullptr) return GNA_ERR_INVALID_ARG;
   if (need_J && n_edges > 0 && J == nullptr) return GNA_ERR_INVALID_ARG;
-  std::set<std::pair<int, int>> seen;
+  std::vector<uint64_t> seen(n_edges > 0 ? n_edges : 0);
   for (int e = 0; e < n_edges; ++e) {
     int a = edges[2 * e], b = edges[2 * e + 1];
     if (a < 0 || a >= n_sites || b < 0 || b >= n_sites || a == b) return GNA_ERR_INVALID_ARG;
-    auto key = std::make_pair(a < b ? a : b, a < b ? b : a);
-    if (!seen.insert(key).second) return GNA_ERR_INVALID_ARG;
+    seen[e] = (uint64_t)(a < b ? a : b) << 32 | (uint32_t)(a < b ? b : a);
     if (need_J && !std::isfinite(J[e])) return GNA_ERR_INVALID_ARG;
   }
+  std::sort(seen.begin(), seen.end());
+  if (std::adjacent_find(seen.begin(), seen.end()) != seen.end()) return GNA_ERR_INVALID_ARG;
   return GNA_OK;
 }
 
@@ -88,6 +90,8 @@ void build(int n, int E, const int32_t* edges, const double* J, int Lmax, HostGr
   h->bond_ent.assign(E, 0);
   h->max_ball.assign(Lmax + 1, 0);
   h->max_span.assign(Lmax + 1, 0);
+  h->bond_info.assign((size_t)E * 32, 0);
+  h->max_pairs.assign(Lmax + 1, 0);
   h->ball_vert.clear();
   h->row_nbr.clear();
   h->nbr_pos.clear();
@@ -116,26 +120,69 @@ void build(int n, int E, const int32_t* edges, const double* J, int Lmax, HostGr
       lo = hi;
       sz[l] = (int)order.size();
     }
-    for (int l = 0; l <= Lmax; ++l) {
-      if (sz[l] > h->max_ball[l]) h->max_ball[l] = sz[l];
-      int span = 0;
-      for (int r = 0; r < sz[l]; ++r) span += h->row_ptr[order[r] + 1] - h->row_ptr[order[r]];
-      if (span > h->max_span[l]) h->max_span[l] = span;
-      h->ball_span[(size_t)e * (Lmax + 1) + l] = span;
+    // the rows' tables: sizes first, then one pass that fills them
+    const int rows = (int)order.size();
+    int ents = 0, npairs = 0;
+    for (int v : order) {
+      const int d = h->row_ptr[v + 1] - h->row_ptr[v];
+      ents += d;
+      npairs += (d + 1) / 2;
     }
-    h->ball_off[e] = (int)h->ball_vert.size();
-    h->bond_ent[e] = (int)h->nbr_pos.size();
-    for (int r = 0; r < (int)order.size(); ++r) {
-      int v = order[r];
-      const int start = (int)h->nbr_pos.size() - h->bond_ent[e];
-      if (start > 0xFFFF) h->pack_ok = false;
-      h->ball_vert.push_back(v);
-      h->row_nbr.push_back((int)h->nbr_pos.size());
-      h->row_pack.push_back(v | ((start & 0xFFFF) << 16));
-      for (int k = h->row_ptr[v]; k < h->row_ptr[v + 1]; ++k) {
-        int u = h->col[k];
-        h->nbr_pos.push_back(pos[u] >= 0 ? pos[u] : INT_MAX);
-        h->nbr_pos16.push_back((int16_t)(pos[u] >= 0 ? pos[u] : 32767));
+    if (e == 0) {  // room for bonds like the first one
+      const size_t R = (size_t)E * rows, N2 = (size_t)E * ents;
+      for (std::vector<int>* v : {&h->ball_vert, &h->row_nbr, &h->row_pack}) v->reserve(R);
+      h->nbr_pos.reserve(N2);
+      h->nbr_pos16.reserve(N2);
+      h->rec.reserve((size_t)E * ((rows + 1) / 2 * 4));
+      h->pairs.reserve((size_t)E * ((npairs + 3) / 4 * 4));
+    }
+    const size_t r0 = h->ball_vert.size(), e0 = h->nbr_pos.size();
+    h->ball_off[e] = (int)r0;
+    h->bond_ent[e] = (int)e0;
+    h->ball_vert.insert(h->ball_vert.end(), order.begin(), order.end());
+    h->row_nbr.resize(r0 + rows);
+    h->row_pack.resize(r0 + rows);
+    h->nbr_pos.resize(e0 + ents);
+    h->nbr_pos16.resize(e0 + ents);
+    const size_t q0 = h->rec.size(), p0 = h->pairs.size();  // 16-byte parts, zero rows as padding
+    h->rec.resize(q0 + (size_t)(rows + 1) / 2 * 4, 0);
+    h->pairs.resize(p0 + (size_t)(npairs + 3) / 4 * 4, 0xFFFFFFFFu);
+    int* info = &h->bond_info[(size_t)e * 32];
+    info[0] = (int)(q0 / 2);
+    info[1] = (int)p0;
+    std::memcpy(info + 2, &h->J[e], sizeof(double));
+    info[4] = edges[2 * e];
+    info[5] = edges[2 * e + 1];
+    int* rec = h->rec.data() + q0;
+    uint32_t* pr = h->pairs.data() + p0;
+    int at = 0, pat = 0, l = 0;
+    for (int r = 0; r < rows; ++r) {
+      const int v = order[r], k0 = h->row_ptr[v], d = h->row_ptr[v + 1] - k0;
+      if (at > 0xFFFF) h->pack_ok = false;
+      h->row_nbr[r0 + r] = (int)e0 + at;
+      h->row_pack[r0 + r] = v | ((at & 0xFFFF) << 16);
+      rec[2 * r] = v | ((d + 1) / 2) << 16;
+      rec[2 * r + 1] = pat;
+      for (int k = 0; k < d; ++k) {
+        const int p = pos[h->col[k0 + k]];
+        h->nbr_pos[e0 + at + k] = p >= 0 ? p : INT_MAX;
+        h->nbr_pos16[e0 + at + k] = (int16_t)(p >= 0 ? p : 32767);
+        // a position as the warp-tiled kernels stage it: 4 p + (p & 1), 0xFFFF when outside
+        const uint32_t s = p < 0 ? 0xFFFFu : (uint32_t)(4 * p + (p & 1));
+        if (k % 2 == 0)
+          pr[pat + k / 2] = s | 0xFFFF0000u;
+        else
+          pr[pat + k / 2] = (pr[pat + k / 2] & 0xFFFFu) | s << 16;
+      }
+      at += d;
+      pat += (d + 1) / 2;
+      for (; l <= Lmax && sz[l] == r + 1; ++l) {
+        h->max_ball[l] = std::max(h->max_ball[l], sz[l]);
+        h->max_span[l] = std::max(h->max_span[l], at);
+        h->ball_span[(size_t)e * (Lmax + 1) + l] = at;
+        h->max_pairs[l] = std::max(h->max_pairs[l], pat);
+        info[8 + l] = sz[l];
+        if (l > 0) info[16 + l] = pat;
       }
     }
     for (int v : order) pos[v] = -1;
@@ -143,19 +190,30 @@ void build(int n, int E, const int32_t* edges, const double* J, int Lmax, HostGr
   h->ball_off[E] = (int)h->ball_vert.size();
 }
 
-template <typename T>
-gna_status upload(gna_graph* g, const std::vector<T>& v, const T** dst) {
-  if (v.empty()) {
+// The handle's arrays in one device allocation, filled by one copy: add() every array, then
+// upload().  (One allocation and copy per array was two thirds of a small graph's creation.)
+struct Packer {
+  std::vector<unsigned char> bytes;
+  std::vector<std::pair<const void**, size_t>> at;  // where each array's device pointer goes, its offset
+  template <typename T>
+  void add(const std::vector<T>& v, const T** dst) {
     *dst = nullptr;
+    if (v.empty()) return;
+    const size_t o = (bytes.size() + 255) / 256 * 256;
+    bytes.resize(o + v.size() * sizeof(T));
+    std::memcpy(bytes.data() + o, v.data(), v.size() * sizeof(T));
+    at.emplace_back((const void**)dst, o);
+  }
+  gna_status upload(gna_graph* g) {
+    if (bytes.empty()) return GNA_OK;
+    void* p = nullptr;
+    GNA_CUDA_TRY(cudaMalloc(&p, bytes.size()));
+    g->allocations.push_back(p);
+    GNA_CUDA_TRY(cudaMemcpy(p, bytes.data(), bytes.size(), cudaMemcpyHostToDevice));
+    for (auto& a : at) *a.first = (const unsigned char*)p + a.second;
     return GNA_OK;
   }
-  void* p = nullptr;
-  GNA_CUDA_TRY(cudaMalloc(&p, v.size() * sizeof(T)));
-  g->allocations.push_back(p);
-  GNA_CUDA_TRY(cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
-  *dst = (const T*)p;
-  return GNA_OK;
-}
+};
 
 }  // namespace
 
@@ -194,32 +252,34 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
   g->d.n = h.n;
   g->d.E = h.E;
   g->d.Lmax = h.Lmax;
-#define UP(vec, field)                       \
-  st = upload(g, vec, &g->d.field);          \
-  if (st != GNA_OK) {                        \
-    gna_graph_destroy(g);                    \
-    return st;                               \
+  Packer pk;
+  pk.add(h.row_ptr, &g->d.row_ptr);
+  pk.add(h.col, &g->d.col);
+  pk.add(h.col_edge, &g->d.col_edge);
+  pk.add(h.wf, &g->d.wf);
+  pk.add(h.wd, &g->d.wd);
+  pk.add(h.edges, &g->d.edges);
+  pk.add(h.J, &g->d.J);
+  pk.add(h.Jz, &g->d.Jz);
+  pk.add(h.hz, &g->d.hz);
+  pk.add(h.cb, &g->d.cb);
+  pk.add(h.ball_off, &g->d.ball_off);
+  pk.add(h.ball_size, &g->d.ball_size);
+  pk.add(h.ball_vert, &g->d.ball_vert);
+  pk.add(h.row_nbr, &g->d.row_nbr);
+  pk.add(h.nbr_pos, &g->d.nbr_pos);
+  pk.add(h.ball_span, &g->d.ball_span);
+  pk.add(h.row_pack, &g->d.row_pack);
+  pk.add(h.nbr_pos16, &g->d.nbr_pos16);
+  pk.add(h.bond_ent, &g->d.bond_ent);
+  pk.add(h.rec, &g->d.rec);
+  pk.add(h.pairs, &g->d.pairs);
+  pk.add(h.bond_info, &g->d.bond_info);
+  st = pk.upload(g);
+  if (st != GNA_OK) {
+    gna_graph_destroy(g);
+    return st;
   }
-  UP(h.row_ptr, row_ptr);
-  UP(h.col, col);
-  UP(h.col_edge, col_edge);
-  UP(h.wf, wf);
-  UP(h.wd, wd);
-  UP(h.edges, edges);
-  UP(h.J, J);
-  UP(h.Jz, Jz);
-  UP(h.hz, hz);
-  UP(h.cb, cb);
-  UP(h.ball_off, ball_off);
-  UP(h.ball_size, ball_size);
-  UP(h.ball_vert, ball_vert);
-  UP(h.row_nbr, row_nbr);
-  UP(h.nbr_pos, nbr_pos);
-  UP(h.ball_span, ball_span);
-  UP(h.row_pack, row_pack);
-  UP(h.nbr_pos16, nbr_pos16);
-  UP(h.bond_ent, bond_ent);
-#undef UP
   g->pack_ok = h.pack_ok;
   g->h_row_ptr = h.row_ptr;
   g->h_col = h.col;
@@ -229,7 +289,12 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
   g->h_J = h.J;
   g->max_ball = h.max_ball;
   g->max_span = h.max_span;
-  for (int v = 0; v < h.n; ++v) g->max_deg = std::max(g->max_deg, h.row_ptr[v + 1] - h.row_ptr[v]);
+  g->max_pairs = h.max_pairs;
+  g->min_deg = h.row_ptr[1] - h.row_ptr[0];
+  for (int v = 0; v < h.n; ++v) {
+    g->max_deg = std::max(g->max_deg, h.row_ptr[v + 1] - h.row_ptr[v]);
+    g->min_deg = std::min(g->min_deg, h.row_ptr[v + 1] - h.row_ptr[v]);
+  }
   *out = g;
   return GNA_OK;
 }
