@@ -5,6 +5,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "dbl.cuh"
 #include "eloc.cuh"
 #include "metro.cuh"
 #include "prop.cuh"
@@ -133,6 +134,16 @@ static gna_status tensor_eloc_run(const TcCall& c, void* ws, size_t ws_bytes, cu
   return tc_run(c, ws, ws_bytes, stream);
 }
 
+// CUDA-core incremental local energy: float64 tanh models on the difference form of dbl.cu
+// where it takes them, the others on the recomputing kernel of simt.cu.
+static gna_status simt_eloc_workspace(const gna_graph* g, const Dims& m, int prec, int64_t B, size_t* bytes) {
+  if (prec == GNA_PREC_FP64) {
+    gna_status st = db_eloc_workspace(g, m, B, bytes);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
+  return simt_workspace(g, m, prec, 2, B, bytes);
+}
+
 static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int op, int64_t B, size_t* bytes) {
   const Dims m = make_dims(g, d);
   const int sp = simt_prec(d);
@@ -144,14 +155,14 @@ static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int 
       return simt_workspace(g, m, sp, 1, B, bytes);
     case GNA_OP_LOCAL_ENERGY_INCREMENTAL:
       if (tensor_prec(d)) return tensor_eloc_workspace(g, m, B, bytes, split_prec(d));
-      return simt_workspace(g, m, sp, 2, B, bytes);
+      return simt_eloc_workspace(g, m, sp, B, bytes);
     case GNA_OP_LOCAL_ENERGY_LOGPSI: {
       // the local-energy call (its own forward gives log Psi), or the two calls in turn
       if (tensor_prec(d)) return tensor_eloc_workspace(g, m, B, bytes, split_prec(d));
       size_t a = 0, b = 0;
       gna_status st = simt_workspace(g, m, sp, 0, B, &a);
       if (st != GNA_OK) return st;
-      st = simt_workspace(g, m, sp, 2, B, &b);
+      st = simt_eloc_workspace(g, m, sp, B, &b);
       if (st != GNA_OK) return st;
       *bytes = a > b ? a : b;
       return GNA_OK;
@@ -159,6 +170,10 @@ static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int 
     case GNA_OP_METROPOLIS: {
       if (tensor_prec(d)) {
         gna_status st = tcm_workspace(g, m, B, bytes);
+        if (st != GNA_ERR_UNSUPPORTED) return st;
+      }
+      if (d->prec == GNA_PREC_FP64) {
+        gna_status st = db_metro_workspace(g, m, B, bytes);
         if (st != GNA_ERR_UNSUPPORTED) return st;
       }
       // the warp sampler propagates tanh differences; ReLU + layer norm takes one chain per CTA
@@ -274,6 +289,10 @@ extern "C" gna_status gna_local_energy(const gna_graph* g, const gna_model_desc*
   sc.B = B;
   sc.eloc = eloc;
   sc.dlogpsi = dlogpsi_bonds;
+  if (d->prec == GNA_PREC_FP64 && mode == GNA_ELOC_INCREMENTAL) {
+    st = db_eloc_run(sc, workspace, workspace_bytes, (cudaStream_t)stream);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
   return simt_run(sc, simt_prec(d), workspace, workspace_bytes, (cudaStream_t)stream);
 }
 
@@ -337,6 +356,12 @@ extern "C" gna_status gna_metropolis_sweep(const gna_graph* g, const gna_model_d
     TcmCall tc{g, sc.m, (const float*)theta, chain_spins, C, n_sweeps, record_every, seed, step0,
                samples_out, logpsi_out, n_accepted, trace};
     return tcm_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
+  }
+  if (d->prec == GNA_PREC_FP64 && !proposal_params) {
+    MetroCall mc{g, sc.m, theta, chain_spins, C, n_sweeps, record_every, seed, step0,
+                 samples_out, logpsi_out, n_accepted, trace, nullptr, 0.0};
+    st = db_metro_run(mc, workspace, workspace_bytes, (cudaStream_t)stream);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
   }
   if (d->act == GNA_ACT_TANH &&
       metro_workspace(g, sc.m, simt_prec(d), C, proposal_params != nullptr, &need) == GNA_OK) {
