@@ -7,8 +7,9 @@
 // counts is the number of FP64 warp instructions and that no SM's pipe stands idle:
 //   - the rows of ball_{l-1} are multiplied instead of those of ball_l (Kagome 2x2x3, L 2: 7 rows
 //     a bond instead of 19);
-//   - tanh(Y + x) - tanh(Y) comes from a rational tanh(x) and the cached E = exp(2Y) with one
-//     reciprocal (about 25 instructions an element; exp, tanh and a division took 70);
+//   - tanh(Y + x) - tanh(Y) comes from a rational tanh(x) and the cached H = tanh Y and 1 - H^2 with
+//     one reciprocal (13 instructions an element, 20 with the updates of H and 1 - H^2 that an
+//     accepted move copies; exp, tanh and a division took 70);
 //   - a warp holds 32 / F rows of F <= 16 features, not one;
 //   - blocks of four warps, so that 1024 chains reach every SM (16 chains a block filled 64 SMs).
 #include <climits>
@@ -23,7 +24,7 @@ namespace {
 
 constexpr int kDbThreads = 128;
 constexpr int kDbWarps = kDbThreads / 32;
-constexpr double kDbCap = 1e140;  // E = exp(2 Y) at most (Y = 161)
+constexpr int kDbBatch = 256;  // bonds of the local energy whose Delta are kept at a time
 
 struct DbArgs {
   DevGraph g;
@@ -31,7 +32,7 @@ struct DbArgs {
   const double* theta;
   int units, uw;      // units per CTA, warps per unit
   int lpr, fpl;       // lanes per row (a power of two), features per lane
-  uint32_t oW, ob, oemb, owr, obr, oav, oz0, olist, ounit;
+  uint32_t oW, ob, oemb, owr, obr, oav, oz0, olist, ores, ounit;
   uint32_t unit_bytes, uz[2], ud, usum, uspin;
   double* ws;
   size_t ws_unit;     // doubles per unit (sampler) or per CTA (local energy)
@@ -60,28 +61,30 @@ struct DbCtx {
 };
 
 __device__ __forceinline__ double db_rcp(double d) {
-  double r;
+  double r;  // about 20 bits; the cubic step leaves 60
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  r = fma(r, fma(-d, r, 1.0), r);
-  return fma(r, fma(-d, r, 1.0), r);
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 __device__ __forceinline__ double db_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
-__device__ __forceinline__ double db_cache(double y) { return fmin(exp(2.0 * y), kDbCap); }
+// H = tanh y and S = 1 - H^2 (its relative precision kept at saturation) from e = exp(-2 |y|).
+__device__ __forceinline__ double2 db_cache(double y) {
+  const double e = exp(-2.0 * fabs(y)), r = db_rcp(1.0 + e);
+  return make_double2(copysign((1.0 - e) * r, y), 4.0 * e * (r * r));
+}
 
-// dH = tanh(Y + x) - tanh(Y) from E = exp(2 Y); NEXT also E' = exp(2 (Y + x)).  tanh(x) = w/Q by a
-// convergent of Lambert's continued fraction: the sixth (relative error 4e-17 up to |x| = 1/4) or
-// the ninth (3e-17 up to 1), chosen for the whole warp.  With c = (1 + E)/2,
-//   dH = E w / (c (Q c + w (c - 1))),  E' = E (Q + w)/(Q - w),
-// the two divisions sharing one reciprocal.  Beyond 1 from exp(-2 |x|), in a form in which
-// nothing cancels or overflows (as el_dtanh_far of eloc.cu).
+// dH = tanh(Y + x) - tanh(Y) = t S/(1 + H t), t = tanh x, from H = tanh Y and S = 1 - H^2; NEXT also
+// the new H and S = S (1 - t^2)/(1 + H t)^2.  t = w/Q by a convergent of Lambert's continued
+// fraction: the sixth (relative error 4e-17 up to |x| = 1/4) or the ninth (3e-17 up to 1), chosen
+// for the whole warp.  Beyond 1 from X = exp(-2 |x|), with 1 + H t summed without cancellation.
 template <bool NEXT>
-__device__ __forceinline__ double db_dtanh(double x, double E, double& Enew) {
+__device__ __forceinline__ double db_dtanh(double x, double2 hs, double2& next) {
   const int hx = __double2hiint(x) & 0x7fffffff;
-  const double z = x * x;
+  const double z = x * x, H = hs.x, S = hs.y;
   double w, Q;
   if (!__any_sync(0xffffffffu, hx > 0x3fd00000)) {
     w = x * fma(z, fma(z, 21.0, 1260.0), 10395.0);
@@ -90,20 +93,15 @@ __device__ __forceinline__ double db_dtanh(double x, double E, double& Enew) {
     w = x * fma(z, fma(z, fma(z, z + 990.0, 135135.0), 4729725.0), 34459425.0);
     Q = fma(z, fma(z, fma(z, fma(z, 45.0, 13860.0), 945945.0), 16216200.0), 34459425.0);
   }
-  const double c = fma(E, 0.5, 0.5);
-  const double den = c * fma(w, c - 1.0, Q * c);
-  double d;
-  if (NEXT) {
-    const double qm = Q - w, r = db_rcp(den * qm);
-    d = E * (w * (r * qm));
-    Enew = E * ((Q + w) * (r * den));
-  } else {
-    d = E * (w * db_rcp(den));
-  }
+  const double r = db_rcp(fma(H, w, Q)), u = S * r;
+  double d = w * u;
+  if (NEXT) next = make_double2(H + d, (u * r) * ((Q - w) * (Q + w)));
   if (hx > 0x3ff00000) {  // (also what is not a number, which stays one)
-    const double X = exp(-2.0 * fabs(x)), s2 = 2.0 * E / (1.0 + E);
-    d = x > 0.0 ? s2 * ((1.0 - X) / fmax(X + E, 1e-300)) : -s2 * ((1.0 - X) / fma(E, X, 1.0));
-    if (NEXT) Enew = x > 0.0 ? E / X : E * X;
+    const double X = exp(-2.0 * fabs(x)), x1 = 1.0 / (1.0 + X), t = copysign((1.0 - X) * x1, x), ah = fabs(H);
+    const double D = (x < 0.0) == (H < 0.0) ? 1.0 + ah * fabs(t) : S / (1.0 + ah) + ah * (2.0 * X * x1);
+    const double v = D > 0.0 ? S / D : 0.0;
+    d = t * v;
+    if (NEXT) next = make_double2(H + d, D > 0.0 ? v / D * (4.0 * X * (x1 * x1)) : S);
     if (x != x) d = x;
   }
   return d;
@@ -162,10 +160,10 @@ __device__ __forceinline__ void db_rowmul(const double* x, const double* W, int 
   }
 }
 
-// Forward of spins sp by `nwarps` warps (this one is `warp`): Y (when Yc) and E of every layer into
-// the cache.  Hb: two row buffers [N][F]; xs: this warp's staging rows [rows_per_warp][2 F].
+// Forward of spins sp by `nwarps` warps (this one is `warp`): Y (when Yc) and (H, 1 - H^2) of every
+// layer into the cache.  Hb: two row buffers [N][F]; xs: this warp's staging rows [rows_per_warp][2 F].
 template <int FPL, typename Sync>
-__device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc, double* Ec, double* Hb, double* xs,
+__device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc, double2* Hc, double* Hb, double* xs,
                                     int warp, int nwarps, Sync sync) {
   const DbArgs& a = *c.a;
   const int N = a.m.N, F = a.m.F, L = a.m.L, R = c.rows_per_warp;
@@ -214,8 +212,9 @@ __device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc
         if (has[j] && v0 + c.row_in_warp < N) {
           const size_t i = ((size_t)(l - 1) * N + v) * F + fs[j];
           if (Yc) Yc[i] = y[j];
-          Ec[i] = db_cache(y[j]);
-          Hn[(size_t)v * F + fs[j]] = tanh(y[j]);
+          const double2 hs = db_cache(y[j]);
+          Hc[i] = hs;
+          Hn[(size_t)v * F + fs[j]] = hs.x;
         }
       }
       __syncwarp();
@@ -229,10 +228,10 @@ __device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc
 }
 
 // Delta log Psi of exchanging the ends of the bond whose record is in `info` (lane i holds int i of
-// DevGraph::bond_info): this warp's lanes' parts of (Re, Im when IM).  NEXT: the rows' new Y and E
-// into the unit's new rows.  uo: byte offset of the unit's shared memory.
+// DevGraph::bond_info): this warp's lanes' parts of (Re, Im when IM).  NEXT: the rows' new Y, H
+// and 1 - H^2 into the unit's new rows.  uo: byte offset of the unit's shared memory.
 template <int FPL, bool NEXT, bool IM, typename Sync>
-__device__ __forceinline__ void db_delta(const DbCtx& c, int info, const int8_t* sp, const double* Yc, const double* Ec,
+__device__ __forceinline__ void db_delta(const DbCtx& c, int info, const int8_t* sp, const double* Yc, const double2* Hc,
                                          double* wsu, uint32_t uo, int uwarp, Sync sync, double& sre, double& sim) {
   const DbArgs& a = *c.a;
   const int N = a.m.N, F = a.m.F, L = a.m.L, R = c.rows_per_warp, uthreads = a.uw * 32;
@@ -282,13 +281,16 @@ __device__ __forceinline__ void db_delta(const DbCtx& c, int info, const int8_t*
 #pragma unroll
       for (int j = 0; j < FPL; ++j) {
         x[j] = fma(av, x[j], zi[min(r, prev) * 2 * F + F + fs[j]]);
-        double En = 0.0;
-        dv[j] = db_dtanh<NEXT>(x[j], Ec[ci + fs[j]], En);
+        double2 nx;
+        dv[j] = db_dtanh<NEXT>(x[j], Hc[ci + fs[j]], nx);
         if (NEXT && ok && has[j]) {
           const double Yn = Yc[ci + fs[j]] + x[j];
-          // far out, where E may have met its cap, from Y itself
-          if ((__double2hiint(Yn) & 0x7fffffff) >= 0x4062c000) En = db_cache(Yn);  // |Y| >= 150
-          reinterpret_cast<double2*>(wsu + a.off_new[l])[(size_t)r * F + fs[j]] = make_double2(Yn, En);
+          // far out, where 1 - H^2 nears the end of the exponents, from Y itself
+          if ((__double2hiint(Yn) & 0x7fffffff) >= 0x4062c000) nx = db_cache(Yn);  // |Y| >= 150
+          double* nw = wsu + a.off_new[l] + ((size_t)r * F + fs[j]) * 3;
+          nw[0] = Yn;
+          nw[1] = nx.x;
+          nw[2] = nx.y;
         }
       }
       if (l == L) {
@@ -345,14 +347,14 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
   };
   double* wsu = a.ws + ((size_t)blockIdx.x * a.units + h) * a.ws_unit;
   const size_t NF = (size_t)N * F;
-  double* Yc = wsu;
-  double* Ec = wsu + L * NF;
+  double2* Hc = (double2*)wsu;
+  double* Yc = wsu + 2 * L * NF;
   const int64_t n_steps = (int64_t)a.n_sweeps * N, rec_steps = (int64_t)a.record_every * N;
   const int64_t n_rec = a.record_every > 0 ? a.n_sweeps / a.record_every : 0;
   for (int64_t ch = (int64_t)blockIdx.x * a.units + h; ch < a.B; ch += (int64_t)gridDim.x * a.units) {
     for (int v = utid; v < N; v += uthreads) sp[v] = a.chain_spins[ch * N + v];
     sync();
-    db_forward<FPL>(c, sp, Yc, Ec, wsu + a.off_h, (double*)(db_smem + uo + a.uz[0]) + (size_t)uwarp * c.rows_per_warp * 2 * F, uwarp,
+    db_forward<FPL>(c, sp, Yc, Hc, wsu + a.off_h, (double*)(db_smem + uo + a.uz[0]) + (size_t)uwarp * c.rows_per_warp * 2 * F, uwarp,
                     a.uw, sync);
     int accepts = 0;
     int64_t base = -32, k = 0, rec = 0;
@@ -388,7 +390,7 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
         const uint64_t u1 = __shfl_sync(0xffffffffu, r1, src);
         const int info = __ldg(a.g.bond_info + (size_t)eb * 32 + lane);
         double dre = 0.0, dim = 0.0;
-        db_delta<FPL, true, false>(c, info, sp, Yc, Ec, wsu, uo, uwarp, sync, dre, dim);
+        db_delta<FPL, true, false>(c, info, sp, Yc, Hc, wsu, uo, uwarp, sync, dre, dim);
         dre = db_sum(dre);
         if (a.uw > 1) {
           if (lane == 0) sum[uwarp] = dre;
@@ -416,13 +418,12 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
           const int* rc = a.g.rec + 2 * (size_t)__shfl_sync(0xffffffffu, info, 0);
           for (int l = 1; l <= L; ++l) {
             const int n = __shfl_sync(0xffffffffu, info, 8 + l) * F;
-            const double2* nw = reinterpret_cast<const double2*>(wsu + a.off_new[l]);
+            const double* nw = wsu + a.off_new[l];
             for (int i = utid; i < n; i += uthreads) {
               const int r = i / F;
               const size_t o = (size_t)(l - 1) * NF + (size_t)(__ldg(rc + 2 * r) & 0xFFFF) * F + (i - r * F);
-              const double2 y = nw[i];
-              Yc[o] = y.x;
-              Ec[o] = y.y;
+              Yc[o] = nw[3 * i];
+              Hc[o] = make_double2(nw[3 * i + 1], nw[3 * i + 2]);
             }
           }
           if (utid == 0) {
@@ -439,11 +440,11 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
         if (a.samples_out)
           for (int v = utid; v < N; v += uthreads) a.samples_out[((size_t)rec * a.B + ch) * N + v] = sp[v];
         if (a.logpsi_out) {
-          const double* YL = Yc + (L - 1) * NF;
+          const double2* HL = Hc + (L - 1) * NF;
           double re = 0.0, im = 0.0;
           for (int i = utid; i < (int)NF; i += uthreads) {
             const int f = i % F;
-            const double hv = tanh(YL[i]);
+            const double hv = HL[i].x;
             re = fma(hv, c.wr[2 * f], re);
             im = fma(hv, c.wr[2 * f + 1], im);
           }
@@ -503,13 +504,13 @@ __global__ void __launch_bounds__(kDbThreads) k_db_eloc(const __grid_constant__ 
       asm volatile("bar.sync %0, %1;" ::"r"(1 + h), "r"(uthreads) : "memory");
   };
   double* wsu = a.ws + (size_t)blockIdx.x * a.ws_unit;
-  double* Ec = wsu;
+  double2* Hc = (double2*)wsu;
   for (int64_t b = blockIdx.x; b < a.B; b += gridDim.x) {
     for (int v = threadIdx.x; v < N; v += kDbThreads) sp[v] = a.spins[b * N + v];
     if (a.dlogpsi)
       for (int e = threadIdx.x; e < E; e += kDbThreads) a.dlogpsi[b * E + e] = 0.f;
     __syncthreads();
-    db_forward<FPL>(c, sp, nullptr, Ec, wsu + a.off_h,
+    db_forward<FPL>(c, sp, nullptr, Hc, wsu + a.off_h,
                     (double*)(db_smem + a.ounit + (size_t)(a.units - 1) * a.unit_bytes + a.ud) + (size_t)warp * c.rows_per_warp * 2 * F,
                     warp, kDbWarps, [] { __syncthreads(); });
     // antiparallel bonds in order, and the diagonal energy
@@ -536,58 +537,57 @@ __global__ void __launch_bounds__(kDbThreads) k_db_eloc(const __grid_constant__ 
       na = all;
       __syncthreads();
     }
-    diag = db_sum(diag);
+    // Delta of up to kDbBatch bonds at a time, then one warp's worth of exponentials for 32 of them
     double er = 0.0, ei = 0.0;
-    if (active)
-      for (int i = h; i < na; i += a.units) {
-        const int e = list[i];
-        const int info = __ldg(a.g.bond_info + (size_t)e * 32 + lane);
-        double dre = 0.0, dim = 0.0;
-        db_delta<FPL, false, true>(c, info, sp, nullptr, Ec, nullptr, uo, uwarp, sync, dre, dim);
-        dre = db_sum(dre);
-        dim = db_sum(dim);
-        if (a.uw > 1) {
-          if (lane == 0) {
-            sum[2 * uwarp] = dre;
-            sum[2 * uwarp + 1] = dim;
+    double2* res = (double2*)(db_smem + a.ores);
+    for (int b0 = 0; b0 < na; b0 += kDbBatch) {
+      const int nb = min(kDbBatch, na - b0);
+      if (active)
+        for (int i = h; i < nb; i += a.units) {
+          const int e = list[b0 + i];
+          const int info = __ldg(a.g.bond_info + (size_t)e * 32 + lane);
+          double dre = 0.0, dim = 0.0;
+          db_delta<FPL, false, true>(c, info, sp, nullptr, Hc, nullptr, uo, uwarp, sync, dre, dim);
+          dre = db_sum(dre);
+          dim = db_sum(dim);
+          if (a.uw > 1) {
+            if (lane == 0) {
+              sum[2 * uwarp] = dre;
+              sum[2 * uwarp + 1] = dim;
+            }
+            sync();
+            dre = dim = 0.0;
+            for (int w = 0; w < a.uw; ++w) {
+              dre += sum[2 * w];
+              dim += sum[2 * w + 1];
+            }
+            sync();
           }
-          sync();
-          dre = dim = 0.0;
-          for (int w = 0; w < a.uw; ++w) {
-            dre += sum[2 * w];
-            dim += sum[2 * w + 1];
-          }
-          sync();
-        }
-        // the terms of 32 bonds wait in the lanes for one exponential
-        if (lane == ((i / a.units) & 31)) {
-          er = dre;
-          ei = dim;
-        }
-        if (a.dlogpsi && uwarp == 0 && lane == 0) a.dlogpsi[b * E + e] = (float)dre;
-        const bool last = i + a.units >= na;
-        if (((i / a.units) & 31) == 31 || last) {
-          const int i0 = i - (((i / a.units) & 31) * a.units), mine = i0 + lane * a.units;
-          double tr = 0.0, ti = 0.0;
-          if (mine <= i && uwarp == 0) {
-            const double amp = exp(er), hJ = 0.5 * __ldg(a.g.J + list[mine]);
-            double sn = 0.0, cs = 1.0;
-            if (ei != 0.0) sincos(ei, &sn, &cs);
-            tr = hJ * (amp * cs);
-            ti = hJ * (amp * sn);
-          }
-          tr = db_sum(tr);
-          ti = db_sum(ti);
-          if (lane == 0 && uwarp == 0) {
-            // sums of earlier batches are kept in shared memory, not in the lanes
-            s_e[kDbWarps + warp] = (i0 == h ? 0.0 : s_e[kDbWarps + warp]) + tr;
-            s_e[2 * kDbWarps + warp] = (i0 == h ? 0.0 : s_e[2 * kDbWarps + warp]) + ti;
+          if (uwarp == 0 && lane == 0) {
+            res[i] = make_double2(dre, dim);
+            if (a.dlogpsi) a.dlogpsi[b * E + e] = (float)dre;
           }
         }
+      __syncthreads();
+      for (int i = threadIdx.x; i < nb; i += kDbThreads) {
+        const double2 d = res[i];
+        const double amp = exp(d.x), hJ = 0.5 * __ldg(a.g.J + list[b0 + i]);
+        double sn = 0.0, cs = 1.0;
+        if (d.y != 0.0) sincos(d.y, &sn, &cs);
+        er += hJ * (amp * cs);
+        ei += hJ * (amp * sn);
       }
+      __syncthreads();
+    }
+    diag = db_sum(diag);
+    if (warp * 32 < na) {  // (warps without a term keep their zeros)
+      er = db_sum(er);
+      ei = db_sum(ei);
+    }
     if (lane == 0) {
       s_e[warp] = diag;
-      if (!active || uwarp != 0 || h >= na) s_e[kDbWarps + warp] = s_e[2 * kDbWarps + warp] = 0.0;
+      s_e[kDbWarps + warp] = er;
+      s_e[2 * kDbWarps + warp] = ei;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -642,6 +642,7 @@ uint64_t db_layout(const gna_graph* g, const Dims& m, bool eloc, int units, int 
   a->oav = take((uint64_t)N * 8);
   a->oz0 = take((uint64_t)2 * F * 8);
   a->olist = eloc ? take((uint64_t)m.E * 2) : 0;
+  a->ores = eloc ? take((uint64_t)kDbBatch * 16) : 0;
   uint64_t zr[2] = {3, 0};
   for (int l = 1; l < L; ++l) {
     const uint64_t rows = (uint64_t)g->max_ball[l] + 1;
@@ -697,12 +698,11 @@ gna_status db_plan(const gna_graph* g, const Dims& m, bool eloc, int64_t B, DbPl
   if (grid > need) grid = need;
   p->grid = (int)(grid < 1 ? 1 : grid);
   const size_t NF = (size_t)m.N * m.F;
-  size_t o = eloc ? m.L * NF : 2 * m.L * NF;  // E, and Y in the sampler
+  size_t o = (eloc ? 2 : 3) * m.L * NF;  // (H, 1 - H^2), and Y in the sampler
   if (!eloc)
     for (int l = 1; l <= m.L; ++l) {
-      o = (o + 1) / 2 * 2;  // (Y, E) pairs
       a.off_new[l] = o;
-      o += (size_t)2 * g->max_ball[l] * m.F;
+      o += (size_t)3 * g->max_ball[l] * m.F;
     }
   a.off_h = o;
   o += 2 * NF;
