@@ -205,6 +205,28 @@ __host__ __device__ inline U64x4 philox4x64_10(uint64_t k0, uint64_t k1, U64x4 c
   return c;
 }
 
+// ---- sums over the per-CTA partials of P values, partial [grid][P] -----------------------------
+// A block of 32 x kSumRows threads sums 32 values: thread (i, r) the CTAs r, r + kSumRows, ..., then
+// the rows in order (fixed order, float64).  One thread per value took 23 us for 152 CTAs -- a
+// chain of loads -- and this 4.
+constexpr int kSumRows = 16;
+#ifdef __CUDACC__
+// value p0 + i of the block, in the threads of row 0
+__device__ inline double sum_partials(const double* partial, int grid, int stride, int p, bool in) {
+  __shared__ double sm[kSumRows][33];
+  const int i = threadIdx.x & 31, r = threadIdx.x >> 5;
+  double s = 0.0;
+  if (in)
+    for (int c = r; c < grid; c += kSumRows) s += partial[(size_t)c * stride + p];
+  sm[r][i] = s;
+  __syncthreads();
+  if (r == 0)
+    for (int k = 1; k < kSumRows; ++k) s += sm[k][i];
+  __syncthreads();
+  return s;
+}
+#endif
+
 // ---- workspace carving --------------------------------------------------------------
 inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
 

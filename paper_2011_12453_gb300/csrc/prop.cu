@@ -245,13 +245,10 @@ __global__ void __launch_bounds__(kPropThreads) k_prop(const PropArgs a) {
 
 // grad = (sum over CTAs of the partials) / count; loss likewise.  Fixed order, float64.
 __global__ void k_prop_reduce(const double* partial, int grid, double* grad, double* loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > kPropParams) return;
-  double s = 0.0, n = 0.0;
-  for (int c = 0; c < grid; ++c) {
-    s += partial[(size_t)c * (kPropParams + 2) + p];
-    n += partial[(size_t)c * (kPropParams + 2) + kPropParams + 1];
-  }
+  const int p = blockIdx.x * 32 + (threadIdx.x & 31);
+  const double s = sum_partials(partial, grid, kPropParams + 2, p, p <= kPropParams);
+  const double n = sum_partials(partial, grid, kPropParams + 2, kPropParams + 1, true);
+  if (threadIdx.x >= 32 || p > kPropParams) return;
   const double inv = n > 0.0 ? 1.0 / n : 0.0;
   if (p < kPropParams)
     grad[p] = s * inv;
@@ -303,7 +300,7 @@ gna_status prop_grad_launch(const gna_graph* g, const int8_t* spins, const float
   GNA_CUDA_TRY(cudaFuncSetAttribute((const void*)k_prop, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   k_prop<<<grid, kPropThreads, smem, st>>>(a);
   GNA_CUDA_TRY(cudaGetLastError());
-  k_prop_reduce<<<(kPropParams + 1 + 255) / 256, 256, 0, st>>>(a.partial, grid, grad, loss);
+  k_prop_reduce<<<(kPropParams + 1 + 31) / 32, 32 * kSumRows, 0, st>>>(a.partial, grid, grad, loss);
   GNA_CUDA_TRY(cudaGetLastError());
   return GNA_OK;
 }

@@ -1158,11 +1158,9 @@ __global__ void __launch_bounds__(kThreadsBwd, 1) k_backward(const SimtArgs<T> a
 
 // grad[p] = sum_cta partial[cta][p], fixed order, float64.
 __global__ void k_reduce_partials(const double* partial, int grid, int P, double* grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  double s = 0.0;
-  for (int c = 0; c < grid; ++c) s += partial[(size_t)c * P + p];
-  grad[p] = s;
+  const int p = blockIdx.x * 32 + (threadIdx.x & 31);
+  const double s = sum_partials(partial, grid, P, p, p < P);
+  if (threadIdx.x < 32 && p < P) grad[p] = s;
 }
 
 // ---------------------------------------------------------------------------------
@@ -1308,7 +1306,7 @@ gna_status simt_launch(const SimtCall& sc, void* ws, size_t ws_bytes, cudaStream
     case OP_BWD:
       k_backward<T><<<p.grid, kThreadsBwd, p.smem, stream>>>(a);
       GNA_CUDA_TRY(cudaGetLastError());
-      k_reduce_partials<<<(sc.m.P + 255) / 256, 256, 0, stream>>>(a.partial, p.grid, sc.m.P, sc.grad);
+      k_reduce_partials<<<(sc.m.P + 31) / 32, 32 * kSumRows, 0, stream>>>(a.partial, p.grid, sc.m.P, sc.grad);
       break;
     default:
       return GNA_ERR_INVALID_ARG;
@@ -1406,7 +1404,7 @@ static gna_status backward_static_launch(const SimtCall& sc, cudaStream_t stream
   a.partial = (double*)w;
   k_backward<T><<<(int)grid, kThreadsBwd, p.smem, stream>>>(a);
   GNA_CUDA_TRY(cudaGetLastError());
-  k_reduce_partials<<<(sc.m.P + 255) / 256, 256, 0, stream>>>(a.partial, (int)grid, sc.m.P, sc.grad);
+  k_reduce_partials<<<(sc.m.P + 31) / 32, 32 * kSumRows, 0, stream>>>(a.partial, (int)grid, sc.m.P, sc.grad);
   GNA_CUDA_TRY(cudaGetLastError());
   return GNA_OK;
 }

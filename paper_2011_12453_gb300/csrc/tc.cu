@@ -2436,10 +2436,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_bwd(const TcbArgs a) {
 }
 
 __global__ void k_tcb_reduce(const double* partial, int grid, int P, double* grad) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= P) return;
-  double s = 0.0;
-  for (int cta = 0; cta < grid; ++cta) s += partial[(size_t)cta * P + p];
+  const int p = blockIdx.x * 32 + (threadIdx.x & 31);
+  const double s = sum_partials(partial, grid, P, p, p < P);
+  if (threadIdx.x >= 32 || p >= P) return;
   grad[p] = s;
   if (!isfinite(s)) atomicOr(&s_tc_status, 2);
 }
@@ -2902,7 +2901,7 @@ static gna_status tcb_launch(const TcbCall& call, void* ws, size_t ws_bytes, siz
   a.partial = (double*)ws;
   k_tc_bwd<<<p.grid, kTcThreads, p.smem, stream>>>(a);
   GNA_CUDA_TRY(cudaGetLastError());
-  k_tcb_reduce<<<(call.m.P + 255) / 256, 256, 0, stream>>>(a.partial, p.grid, call.m.P, call.grad);
+  k_tcb_reduce<<<(call.m.P + 31) / 32, 32 * kSumRows, 0, stream>>>(a.partial, p.grid, call.m.P, call.grad);
   GNA_CUDA_TRY(cudaGetLastError());
   return GNA_OK;
 }
