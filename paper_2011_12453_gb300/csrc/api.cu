@@ -121,26 +121,24 @@ namespace gna {
 // shared memory, else (and in BF16) on the tensor-memory kernel.
 static gna_status tensor_eloc_workspace(const gna_graph* g, const Dims& m, int64_t B, size_t* bytes, int split) {
   if (split) {
-    gna_status st = el_workspace(g, m, B, bytes);
+    gna_status st = el_workspace(g, m, B, false, bytes);
     if (st != GNA_ERR_UNSUPPORTED) return st;
   }
   return tc_workspace(g, m, TC_ELOC, B, bytes, split);
 }
 static gna_status tensor_eloc_run(const TcCall& c, void* ws, size_t ws_bytes, cudaStream_t stream) {
   if (c.split) {
-    gna_status st = el_run(c, ws, ws_bytes, stream);
+    gna_status st = el_run(c, false, ws, ws_bytes, stream);
     if (st != GNA_ERR_UNSUPPORTED) return st;
   }
   return tc_run(c, ws, ws_bytes, stream);
 }
 
-// CUDA-core incremental local energy: float64 tanh models on the difference form of dbl.cu
-// where it takes them, the others on the recomputing kernel of simt.cu.
+// FP32 and FP64 incremental local energy: the difference forms of eloc_impl.cuh and dbl.cu where
+// they take the model, else the recomputing kernel of simt.cu.
 static gna_status simt_eloc_workspace(const gna_graph* g, const Dims& m, int prec, int64_t B, size_t* bytes) {
-  if (prec == GNA_PREC_FP64) {
-    gna_status st = db_eloc_workspace(g, m, B, bytes);
-    if (st != GNA_ERR_UNSUPPORTED) return st;
-  }
+  gna_status st = prec == GNA_PREC_FP64 ? db_eloc_workspace(g, m, B, bytes) : el_workspace(g, m, B, true, bytes);
+  if (st != GNA_ERR_UNSUPPORTED) return st;
   return simt_workspace(g, m, prec, 2, B, bytes);
 }
 
@@ -289,8 +287,10 @@ extern "C" gna_status gna_local_energy(const gna_graph* g, const gna_model_desc*
   sc.B = B;
   sc.eloc = eloc;
   sc.dlogpsi = dlogpsi_bonds;
-  if (d->prec == GNA_PREC_FP64 && mode == GNA_ELOC_INCREMENTAL) {
-    st = db_eloc_run(sc, workspace, workspace_bytes, (cudaStream_t)stream);
+  if (mode == GNA_ELOC_INCREMENTAL) {
+    const TcCall tc{g, m, TC_ELOC, (const float*)theta, spins, B, nullptr, eloc, dlogpsi_bonds, 0};
+    st = d->prec == GNA_PREC_FP64 ? db_eloc_run(sc, workspace, workspace_bytes, (cudaStream_t)stream)
+                                  : el_run(tc, true, workspace, workspace_bytes, (cudaStream_t)stream);
     if (st != GNA_ERR_UNSUPPORTED) return st;
   }
   return simt_run(sc, simt_prec(d), workspace, workspace_bytes, (cudaStream_t)stream);

@@ -84,15 +84,21 @@ __device__ __forceinline__ void split3(uint64_t m1, float a, float b, uint32_t& 
 // B fragments of W (2F x F, row-major float32, rounded to BF16), FC = F / 16: entry
 // ((kc * FC + c) * 32 + lane) holds, for K step kc (16 rows of W) and output chunk c, the
 // registers (b0, b1) of column tile 2c and (b0, b1) of column tile 2c + 1.
+// term: 0 = bf16(w), 1 = bf16 of what that leaves, 2 = bf16 of what both leave.
+__device__ __forceinline__ float wterm(float w, int term) {
+  for (int t = 0; t < term; ++t) w -= __bfloat162float(__float2bfloat16_rn(w));
+  return w;
+}
 template <int FC>
-__device__ __forceinline__ uint4 make_wfrag(const float* W, int kc, int c, int lane) {
+__device__ __forceinline__ uint4 make_wfrag(const float* W, int kc, int c, int lane, int term) {
   constexpr int F = 16 * FC;
   const int n = lane >> 2, q = lane & 3;
   uint32_t r[4];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float* w = W + (size_t)(16 * kc + 4 * q) * F + 16 * c + 4 * (n >> 1) + 2 * h + (n & 1);
-    const __nv_bfloat162 x = __floats2bfloat162_rn(w[0], w[F]), y = __floats2bfloat162_rn(w[2 * F], w[3 * F]);
+    const __nv_bfloat162 x = __floats2bfloat162_rn(wterm(w[0], term), wterm(w[F], term));
+    const __nv_bfloat162 y = __floats2bfloat162_rn(wterm(w[2 * F], term), wterm(w[3 * F], term));
     r[2 * h] = *reinterpret_cast<const uint32_t*>(&x);
     r[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&y);
   }

@@ -5,7 +5,8 @@ that end on, just before and just after a multiple of 16 rows, one layer and eig
 that units swing further than the tanh series reaches.
 
 Tolerance: the derived bound on each Delta and each sample of tests/bounds.py, plus the float32
-rounding of the returned Delta and of each term, as for the other local-energy tests."""
+rounding of the returned Delta and of each term, as for the other local-energy tests.  The same
+tiles in FP32 (tanh, and ReLU + layer norm): 1e-5 of the terms' magnitude (tests/scales.py)."""
 import numpy as np
 import pytest
 
@@ -13,6 +14,7 @@ from oracle import gcn, heisenberg as hz
 from paper_2011_12453_gb300 import build as B, gna, workloads as W
 
 import bounds as BD
+import scales as SC
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +90,30 @@ def test_bonds_without_antiparallel_partners(torch):
     _, _, eb = BD.bond_bounds(th, 32, 3, Ah, g.edges, g.J, s[1:2], "bf16x2")
     want = hz.local_energy(lambda x: gcn.logpsi_complex(th, 32, 3, Ah, x), g.edges, g.J, s[1:2])
     assert abs(E[1, 0] + 1j * E[1, 1] - want[0]) <= eb[0] + 2.0 ** -21 * 0.25 * g.J.sum()
+
+
+@pytest.mark.parametrize("act", ["tanh", "relu_ln"])
+@pytest.mark.parametrize("name,F,L,scale", [("two", 16, 1, 0.3), ("ring40", 16, 8, 0.3), ("ring40", 32, 7, 0.3),
+                                            ("isolated", 64, 3, 0.3), ("complete9", 32, 2, 0.3), ("bipartite", 48, 3, 0.1),
+                                            ("kagome3", 64, 3, 0.3), ("kagome3", 16, 3, 1.0), ("tri5", 48, 2, 0.3),
+                                            ("er30", 32, 4, 0.3)])
+def test_fp32_tiles_against_the_oracle(torch, name, F, L, scale, act):
+    g = GRAPHS[name]()
+    one = np.ones(g.n_edges)
+    xxz = (one, -0.7 * one, 0.5 * one, 0.25 * one) if act == "relu_ln" else None
+    theta = torch.tensor(W.random_theta(F, L, seed=F + L, scale=scale), dtype=torch.float32, device="cuda")
+    th = theta.double().cpu().numpy()
+    graph = gna.Graph(g.n_sites, g.edges, g.J, L, xxz=xxz)
+    model = gna.Model(F, L, gna.PREC_FP32, act=gna.ACT_RELU_LN if act == "relu_ln" else gna.ACT_TANH)
+    Ah = gcn.norm_adjacency(gcn.adjacency(g.n_sites, g.edges))
+    s = W.random_spins(g.n_sites, 7, seed=3)
+    E, dl = gna.local_energy(graph, model, theta, torch.tensor(s, device="cuda"), gna.ELOC_INCREMENTAL, bonds=True)
+    psi = lambda x: gcn.logpsi_complex(th, F, L, Ah, x, True, act)  # noqa: E731
+    kw = {"xxz": xxz} if xxz is not None else {}
+    want = hz.local_energy(psi, g.edges, g.J, s, **kw)
+    err = np.abs(E.cpu().numpy()[:, 0] + 1j * E.cpu().numpy()[:, 1] - want)
+    assert np.all(err <= 1e-5 * np.maximum(SC.eloc_scale(th, F, L, Ah, g.edges, g.J, s, act=act, **kw), 1.0)), err
+    d = hz.bond_log_ratios(psi, g.edges, s)
+    want_d = np.where(np.isnan(d.real), 0.0, d.real)
+    lim = 1e-5 * np.maximum(SC.delta_scale(th, F, L, Ah, g.edges, s, act=act), 1.0) + 2.0 ** -24 * np.abs(want_d)
+    assert np.all(np.abs(dl.cpu().numpy() - want_d) <= lim), np.max(np.abs(dl.cpu().numpy() - want_d) - lim)
