@@ -240,6 +240,7 @@ struct Plan {
   int G = 1;               // bonds processed together (local energy)
   int partial_in_smem = 0; // backward: per-CTA gradient partial in shared memory
   int prop_rows = 0;       // Metropolis with a proposal network: row buffer capacity
+  int threads = 0;         // threads per CTA
 };
 
 }  // namespace gna

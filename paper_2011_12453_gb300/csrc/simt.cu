@@ -975,7 +975,11 @@ __global__ void __launch_bounds__(kThreads) k_metropolis(const SimtArgs<T> a) {
   }
 }
 
-// Reverse mode of Eq. (gcn) and the readout; activations recomputed per sample.
+// Reverse mode of Eq. (gcn) and the readout; activations recomputed per sample.  512 threads an
+// SM (128 registers each), as four blocks of 128, two of 256 or one of 512 threads, the smallest
+// whose features fit shared memory: the phases of a small sample occupy few threads (2F F / 4 of
+// them in dW), and other samples' blocks fill in.  FP64 Kagome 2x2x3, F 16, 1024 samples: 245 us with
+// one block an SM.
 constexpr int kThreadsBwd = 512;
 
 template <typename T>
@@ -1225,10 +1229,16 @@ gna_status simt_plan(const gna_graph* g, const Dims& m, int op, int64_t B, Plan*
     p->region_in_smem = 0;
     p->smem = (int)out.total;
   }
+  p->threads = kThreads;
+  if (op == OP_BWD) {
+    int blocks = 4;
+    while (blocks > 1 && (size_t)blocks * (p->smem + 2048) > (size_t)di.smem_optin) blocks /= 2;
+    p->threads = kThreadsBwd / blocks;
+  }
   const void* kp = kernel_ptr<T>(op);
   GNA_CUDA_TRY(cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
   int occ = 0;
-  GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, op == OP_BWD ? kThreadsBwd : kThreads, p->smem));
+  GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, p->threads, p->smem));
   if (occ < 1) occ = 1;
   int64_t grid = (int64_t)di.sms * occ;
   if (B < grid) grid = B;
@@ -1304,7 +1314,7 @@ gna_status simt_launch(const SimtCall& sc, void* ws, size_t ws_bytes, cudaStream
       k_metropolis<T><<<p.grid, kThreads, p.smem, stream>>>(a);
       break;
     case OP_BWD:
-      k_backward<T><<<p.grid, kThreadsBwd, p.smem, stream>>>(a);
+      k_backward<T><<<p.grid, p.threads, p.smem, stream>>>(a);
       GNA_CUDA_TRY(cudaGetLastError());
       k_reduce_partials<<<(sc.m.P + 31) / 32, 32 * kSumRows, 0, stream>>>(a.partial, p.grid, sc.m.P, sc.grad);
       break;
@@ -1402,7 +1412,7 @@ static gna_status backward_static_launch(const SimtCall& sc, cudaStream_t stream
     w += align_up((size_t)grid * region_bytes);
   }
   a.partial = (double*)w;
-  k_backward<T><<<(int)grid, kThreadsBwd, p.smem, stream>>>(a);
+  k_backward<T><<<(int)grid, p.threads, p.smem, stream>>>(a);
   GNA_CUDA_TRY(cudaGetLastError());
   k_reduce_partials<<<(sc.m.P + 31) / 32, 32 * kSumRows, 0, stream>>>(a.partial, (int)grid, sc.m.P, sc.grad);
   GNA_CUDA_TRY(cudaGetLastError());
