@@ -304,39 +304,6 @@ def run_reference(a):
 # our arm
 # ---------------------------------------------------------------------------------
 
-# DRAM bytes per sample of the dominant kernels from one ncu capture (dram__bytes_read.sum +
-# dram__bytes_write.sum of one launch / the samples it processed), valid only for the source file
-# that was profiled: keyed by (workload, kernel) with the SHA-256 of that source (carried
-# forward only across changes to other kernels of the file).
-PROFILED_TRAFFIC = {
-    # ncu --set full of gna_local_energy_logpsi, 2048 configurations, one launch: 3,085,824 B read
-    # + 1,172,992 B written
-    ("kagome_6x6x3_heisenberg", "k_tc<1>"): {"bytes_per_unit": (3085824 + 1172992) / 2048,
-                                             "sha256": "4f986c229ef99251b5f5cf6d28437d630522986576258425c1c822240624057c"},
-    # the same for BF16 operands: 3,069,952 B read + 1,056,768 B written
-    ("kagome_6x6x3_heisenberg", "k_tc<0>"): {"bytes_per_unit": (3069952 + 1056768) / 2048,
-                                             "sha256": "4f986c229ef99251b5f5cf6d28437d630522986576258425c1c822240624057c"},
-    # ncu --set full, 2048 chains, one sweep: 481,241,600 B read + 1,433,287,424 B written (the
-    # sampler's code is unchanged since; the file changed in the local-energy kernel only)
-    ("kagome_6x6x3_heisenberg", "k_tc_metro"): {"bytes_per_unit": (481241600 + 1433287424) / 2048,
-                                                "sha256": "4f986c229ef99251b5f5cf6d28437d630522986576258425c1c822240624057c"},
-}
-
-
-def _source_sha(rel):
-    import hashlib
-
-    with open(os.path.join(ROOT, "paper_2011_12453_gb300", "csrc", rel), "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()
-
-
-def profiled_traffic(workload, kernel, source, units):
-    rec = PROFILED_TRAFFIC.get((workload, kernel))
-    if rec is None or rec["sha256"] != _source_sha(source):
-        return None
-    return rec["bytes_per_unit"] * units
-
-
 def sweep_flops(g, F, L, ball, deg_of, spins_np, steps_per_chain):
     """Expected algorithmic FLOPs of `steps_per_chain` plain exchange proposals per chain: the
     bond is uniform over the edges, an antiparallel bond costs
@@ -441,7 +408,7 @@ def measure_workload(key, prec_name, dev, flush, K_timed, peaks, peak_kind):
                                      "backward_sgd": float(ph[:, 2].mean())},
             "eloc_samples_per_s": Bn / (t_eloc / 1000.0),
             "sample_updates_per_s": Bn / (upd / 1000.0),
-            "roofline": {"bound": "tensor", "kernel": "k_tc (gna_local_energy_logpsi, %s)" % prec_name,
+            "roofline": {"bound": "tensor", "kernel": "%s (gna_local_energy_logpsi, %s)" % ("k_eloc" if prec == gna.PREC_BF16X2 else "k_tc", prec_name),
                          "achieved": achieved, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                          "frac": achieved / peaks["bf16_tflops_sustained"],
                          "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl,
@@ -608,9 +575,9 @@ def run_ours(a):
         if prec in (gna.PREC_BF16, gna.PREC_BF16X2) and prop is None:
             roof = {"bound": "tensor", "achieved": fl_sweep / (t_sweep / 1000.0) / 1e12,
                     "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
-                    "kernel": "k_tc_metro (gna_metropolis_sweep, %d sweeps, BF16 tcgen05)" % S,
+                    "kernel": "k_mt_metro (gna_metropolis_sweep, %d sweeps, BF16 mma.sync)" % S,
                     "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl_sweep,
-                    "traffic": profiled_traffic(wl["workload"], "k_tc_metro", "tc.cu", C * S)}
+                    "traffic": None}
         else:
             roof = {"bound": "alu", "achieved": fl_sweep / (t_sweep / 1000.0) / 1e12, "peak": alu_peak,
                     "unit": "TFLOP/s", "kernel": "k_metro_warp (gna_metropolis_sweep, %d sweeps)" % S,
@@ -619,14 +586,13 @@ def run_ours(a):
     elif prec in (gna.PREC_BF16, gna.PREC_BF16X2):
         roof = {"bound": "tensor", "achieved": fl_incr / (t_incr / 1000.0) / 1e12,
                 "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
-                "kernel": ("k_tc<1> (gna_local_energy_logpsi, split BF16 operands, tcgen05)"
+                "kernel": ("k_eloc (gna_local_energy_logpsi, split BF16 operands, mma.sync)"
                            if prec == gna.PREC_BF16X2 else "k_tc<0> (gna_local_energy_logpsi, BF16 tcgen05)"),
                 "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl_incr,
-                "traffic": profiled_traffic(wl["workload"], "k_tc<1>" if prec == gna.PREC_BF16X2 else "k_tc<0>",
-                                            "tc.cu", Bn)}
+                "traffic": None}
     else:
         roof = {"bound": "alu", "achieved": fl_incr / (t_incr / 1000.0) / 1e12, "peak": alu_peak,
-                "unit": "TFLOP/s", "kernel": "k_eloc_incr (gna_local_energy incremental, FP32)",
+                "unit": "TFLOP/s", "kernel": "k_eloc (gna_local_energy incremental, FP32)",
                 "peak_source": "derived: 152 SM x 128 FP32 lanes x 2 x sm_max_mhz", "flops_per_launch": fl_incr,
                 "traffic": None}
     roof["frac"] = roof["achieved"] / roof["peak"]
@@ -684,7 +650,7 @@ def run_ours(a):
             # per step: the sweep, then per update the local energy with log Psi (one launch on the
             # tensor cores, forward + local energy otherwise), 4 weight kernels, backward + its
             # reduction, SGD
-            "gpu_launches": int(Ksteps * (1 + (8 if prec in (gna.PREC_BF16, gna.PREC_BF16X2) else 9) * K)),
+            "gpu_launches": int(Ksteps * (1 + (6 if prec in (gna.PREC_BF16, gna.PREC_BF16X2) else 7) * K)),
             "clocks": clk,
             "acceptance": float(acc.sum().item()) / max(1, state["step"] * S * C * N),
         }

@@ -8,6 +8,7 @@
 #include "dbl.cuh"
 #include "eloc.cuh"
 #include "metro.cuh"
+#include "mtile.cuh"
 #include "prop.cuh"
 #include "tc.cuh"
 
@@ -167,7 +168,7 @@ static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int 
     }
     case GNA_OP_METROPOLIS: {
       if (tensor_prec(d)) {
-        gna_status st = tcm_workspace(g, m, B, bytes);
+        gna_status st = mt_workspace(g, m, B, bytes);
         if (st != GNA_ERR_UNSUPPORTED) return st;
       }
       if (d->prec == GNA_PREC_FP64) {
@@ -349,13 +350,13 @@ extern "C" gna_status gna_metropolis_sweep(const gna_graph* g, const gna_model_d
   sc.trace = trace;
   sc.prop = proposal_params;
   sc.prop_eps = proposal_eps;
-  // BF16 models, plain moves: the tensor-core sampler; otherwise the warp-per-chain sampler
-  // when the model fits it, else one chain per CTA
-  size_t need = 0;
-  if (tensor_prec(d) && !proposal_params && tcm_workspace(g, sc.m, C, &need) == GNA_OK) {
-    TcmCall tc{g, sc.m, (const float*)theta, chain_spins, C, n_sweeps, record_every, seed, step0,
-               samples_out, logpsi_out, n_accepted, trace};
-    return tcm_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
+  // plain moves of BF16 models: a warp per chain on the matrix units; otherwise the warp-per-chain
+  // samplers when the model fits them, else one chain per CTA
+  if (tensor_prec(d) && !proposal_params) {
+    MetroCall mc{g, sc.m, theta, chain_spins, C, n_sweeps, record_every, seed, step0,
+                 samples_out, logpsi_out, n_accepted, trace, nullptr, 0.0};
+    st = mt_run(mc, workspace, workspace_bytes, (cudaStream_t)stream);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
   }
   if (d->prec == GNA_PREC_FP64 && !proposal_params) {
     MetroCall mc{g, sc.m, theta, chain_spins, C, n_sweeps, record_every, seed, step0,
@@ -363,6 +364,7 @@ extern "C" gna_status gna_metropolis_sweep(const gna_graph* g, const gna_model_d
     st = db_metro_run(mc, workspace, workspace_bytes, (cudaStream_t)stream);
     if (st != GNA_ERR_UNSUPPORTED) return st;
   }
+  size_t need = 0;
   if (d->act == GNA_ACT_TANH &&
       metro_workspace(g, sc.m, simt_prec(d), C, proposal_params != nullptr, &need) == GNA_OK) {
     MetroCall mc{g, sc.m, theta, chain_spins, C, n_sweeps, record_every, seed, step0,
