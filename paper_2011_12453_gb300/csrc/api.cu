@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include "dbl.cuh"
 #include "eloc.cuh"
+#include "fwd.cuh"
 #include "metro.cuh"
 #include "mtile.cuh"
 #include "prop.cuh"
@@ -135,6 +136,22 @@ static gna_status tensor_eloc_run(const TcCall& c, void* ws, size_t ws_bytes, cu
   return tc_run(c, ws, ws_bytes, stream);
 }
 
+// Tensor-core forward: the same choice.
+static gna_status tensor_forward_workspace(const gna_graph* g, const Dims& m, int64_t B, size_t* bytes, int split) {
+  if (split) {
+    gna_status st = fx_workspace(g, m, B, bytes);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
+  return tc_workspace(g, m, TC_FWD, B, bytes, split);
+}
+static gna_status tensor_forward_run(const TcCall& c, void* ws, size_t ws_bytes, cudaStream_t stream) {
+  if (c.split) {
+    gna_status st = fx_run(c.g, c.m, c.theta, c.spins, c.B, c.logpsi, ws, ws_bytes, stream);
+    if (st != GNA_ERR_UNSUPPORTED) return st;
+  }
+  return tc_run(c, ws, ws_bytes, stream);
+}
+
 // FP32 and FP64 incremental local energy: the difference forms of eloc_impl.cuh and dbl.cu where
 // they take the model, else the recomputing kernel of simt.cu.
 static gna_status simt_eloc_workspace(const gna_graph* g, const Dims& m, int prec, int64_t B, size_t* bytes) {
@@ -148,7 +165,7 @@ static gna_status op_workspace(const gna_graph* g, const gna_model_desc* d, int 
   const int sp = simt_prec(d);
   switch (op) {
     case GNA_OP_FORWARD:
-      if (tensor_prec(d)) return tc_workspace(g, m, TC_FWD, B, bytes, split_prec(d));
+      if (tensor_prec(d)) return tensor_forward_workspace(g, m, B, bytes, split_prec(d));
       return simt_workspace(g, m, sp, 0, B, bytes);
     case GNA_OP_LOCAL_ENERGY_FULL:
       return simt_workspace(g, m, sp, 1, B, bytes);
@@ -248,7 +265,7 @@ extern "C" gna_status gna_forward(const gna_graph* g, const gna_model_desc* d, c
   const Dims m = make_dims(g, d);
   if (tensor_prec(d)) {
     TcCall tc{g, m, TC_FWD, (const float*)theta, spins, B, logpsi, nullptr, nullptr, split_prec(d)};
-    return tc_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
+    return tensor_forward_run(tc, workspace, workspace_bytes, (cudaStream_t)stream);
   }
   SimtCall sc{};
   sc.g = g;

@@ -177,3 +177,22 @@ def test_proposal_gradient(torch, name, n, n_up):
     want_loss, want = P.loss_and_grad(p32.double().cpu().numpy(), phi, tgt)
     assert abs(loss.item() - want_loss) <= 1e-4 * abs(want_loss)
     np.testing.assert_allclose(grad.cpu().numpy(), want, rtol=0, atol=1e-4 * np.abs(want).max())
+
+
+@pytest.mark.parametrize("name,F,L,n", [("two", 16, 1, 1), ("isolated", 64, 3, 5), ("ring40", 48, 2, 153), ("kagome6", 32, 4, 1),
+                                        ("kagome6", 64, 2, 700), ("tri14", 64, 2, 400), ("bipartite", 16, 3, 17)])
+def test_bf16x2_forward(torch, name, F, L, n):
+    # against the forward inside the local energy (the same sums: equal), and on a few
+    # configurations against the oracle: 2^-16 operands, some hundred sites, as the other forward tests
+    g = GRAPHS[name]()
+    theta = torch.tensor(W.random_theta(F, L, seed=F, scale=0.3), dtype=torch.float32, device="cuda")
+    graph, model = gna.Graph.from_workload(g, L), gna.Model(F, L, gna.PREC_BF16X2)
+    s = W.random_spins(g.n_sites, n, seed=9)
+    st = torch.tensor(s, device="cuda")
+    lp = gna.forward(graph, model, theta, st)
+    assert torch.equal(lp, gna.local_energy_logpsi(graph, model, theta, st)[1])
+    th = theta.double().cpu().numpy()
+    w = slice(3 * F, 3 * F + 2 * F * F)
+    th[w] = bf16_round(th[w])
+    want = gcn.logpsi(th, F, L, gcn.norm_adjacency(gcn.adjacency(g.n_sites, g.edges)), s[-3:])
+    assert np.abs(lp[-3:].cpu().numpy() - want).max() <= 2e-4 * max(1.0, np.abs(want).max())
