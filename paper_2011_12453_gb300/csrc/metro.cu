@@ -19,6 +19,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "frag.cuh"
 #include "metro.cuh"
 #include "prop.cuh"
 
@@ -104,13 +105,17 @@ __device__ __forceinline__ T wsum(T v) {
 // e = exp(-2|y|); falls back to the direct difference when 1 + H t is small (a unit
 // swinging across saturation, where dH is O(1) and the difference has no cancellation).
 template <typename T>
+__device__ __noinline__ T dtanh_far(T y, T dy) {
+  return m_tanh(y + dy) - m_tanh(y);
+}
+template <typename T>
 __device__ __forceinline__ T dtanh(T y, T dy) {
   const T e = m_exp((T)-2 * fabs(y));
   const T t = m_tanh(dy);
   const T sg = y < (T)0 ? (T)-1 : (T)1;
   const T ope = (T)1 + e;
   const T den = ope * (ope + sg * ((T)1 - e) * t);
-  return den > (T)1e-3 ? m_div((T)4 * e * t, den) : m_tanh(y + dy) - m_tanh(y);
+  return den > (T)1e-3 ? m_div((T)4 * e * t, den) : dtanh_far(y, dy);
 }
 
 template <typename T>
@@ -191,18 +196,39 @@ __device__ void pair_phi(const DevGraph& g, const int8_t* sp, int i, int j, int 
   f[8] = cj ? bj / (T)cj : (T)0;
 }
 
+// Sums of two products in the roundings that these logits have always had.
+__device__ __forceinline__ float m_dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ double m_dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+__device__ __forceinline__ float m_dot2_last(float a, float b, float c, float d) {
+  return __fmaf_rn(c, d, __fmul_rn(a, b));
+}
+__device__ __forceinline__ double m_dot2_last(double a, double b, double c, double d) {
+  return __fma_rn(c, d, __dmul_rn(a, b));
+}
+template <typename T>
+__device__ __noinline__ T m_tanh_call(T x) {
+  return m_tanh(x);
+}
+
 // Logits of rows r < n of (rc[r] -> ro[r]) evaluated in the state selected by rx[r]
 // (0: s, 1: s with (pa, pb) exchanged).  Returns the logit of row `lane` (and row lane+32).
+// Four rows (float32) share the loads of the weights.  Not inlined (nor what else the proposal calls): a
+// step passes through all of the kernel's code, which has to stay in the instruction caches.
 template <typename T>
-__device__ void warp_logits(const DevGraph& g, const int8_t* sp, const T* P, const int* rc, const int* ro,
-                            const int* rx, int n, int pa, int pb, T* out0, T* out1) {
+struct Logits {
+  T lg0, lg1;
+};
+template <typename T>
+__device__ __noinline__ Logits<T> warp_logits(const DevGraph& g, const int8_t* sp, const T* P, const int* rc,
+                                              const int* ro, const int* rx, int n, int pa, int pb) {
+  constexpr int kLogitRows = sizeof(T) == 4 ? 4 : 1;  // at a time; float64 has no registers for more
   const int lane = threadIdx.x & 31;
   const T* W1 = P + kPropOW1;
   const T* b1 = P + kPropOb1;
   const T* W2 = P + kPropOW2;
   const T* b2 = P + kPropOb2;
   const T* w3 = P + kPropOw3;
-  T lg0 = 0, lg1 = 0;
+  Logits<T> out{0, 0};
   for (int base = 0; base < n; base += 32) {
     T f[kPropIn];
     const int r = base + lane;
@@ -213,41 +239,55 @@ __device__ void warp_logits(const DevGraph& g, const int8_t* sp, const T* P, con
       for (int q = 0; q < kPropIn; ++q) f[q] = 0;
     }
     const int cnt = min(32, n - base);
-    for (int rr = 0; rr < cnt; ++rr) {
-      // hidden layer 1 (units lane, lane + 32) of row base + rr
-      T z0 = b1[lane], z1 = b1[lane + 32];
+    for (int rr = 0; rr < cnt; rr += kLogitRows) {
+      // hidden layer 1 (units lane, lane + 32) of rows base + rr ..
+      T h0[kLogitRows], h1[kLogitRows], y0[kLogitRows], y1[kLogitRows];
 #pragma unroll
-      for (int q = 0; q < kPropIn; ++q) {
-        const T x = __shfl_sync(0xffffffffu, f[q], rr);
-        z0 += x * W1[q * kPropHid + lane];
-        z1 += x * W1[q * kPropHid + lane + 32];
+      for (int i = 0; i < kLogitRows; ++i) {
+        T z0 = b1[lane], z1 = b1[lane + 32];
+#pragma unroll
+        for (int q = 0; q < kPropIn; ++q) {
+          const T x = __shfl_sync(0xffffffffu, f[q], rr + i);
+          z0 += x * W1[q * kPropHid + lane];
+          z1 += x * W1[q * kPropHid + lane + 32];
+        }
+        h0[i] = m_tanh_call(z0);
+        h1[i] = m_tanh_call(z1);
+        y0[i] = b2[lane];
+        y1[i] = b2[lane + 32];
       }
-      const T h0 = m_tanh(z0), h1 = m_tanh(z1);
       // hidden layer 2
-      T y0 = b2[lane], y1 = b2[lane + 32];
+#pragma unroll 2
       for (int q = 0; q < 32; ++q) {
-        const T xa = __shfl_sync(0xffffffffu, h0, q);
-        const T xb = __shfl_sync(0xffffffffu, h1, q);
-        y0 += xa * W2[q * kPropHid + lane] + xb * W2[(q + 32) * kPropHid + lane];
-        y1 += xa * W2[q * kPropHid + lane + 32] + xb * W2[(q + 32) * kPropHid + lane + 32];
+        const T wa0 = W2[q * kPropHid + lane], wb0 = W2[(q + 32) * kPropHid + lane];
+        const T wa1 = W2[q * kPropHid + lane + 32], wb1 = W2[(q + 32) * kPropHid + lane + 32];
+#pragma unroll
+        for (int i = 0; i < kLogitRows; ++i) {
+          const T xa = __shfl_sync(0xffffffffu, h0[i], q);
+          const T xb = __shfl_sync(0xffffffffu, h1[i], q);
+          y0[i] += m_dot2(xa, wa0, xb, wb0);
+          y1[i] += m_dot2(xa, wa1, xb, wb1);
+        }
       }
-      T z = m_tanh(y0) * w3[lane] + m_tanh(y1) * w3[lane + 32];
-      z = wsum(z) + P[kPropOb3];
-      if (lane == rr) {
-        if (base == 0)
-          lg0 = z;
-        else
-          lg1 = z;
+#pragma unroll
+      for (int i = 0; i < kLogitRows; ++i) {
+        T z = m_dot2_last(m_tanh_call(y0[i]), w3[lane], m_tanh_call(y1[i]), w3[lane + 32]);
+        z = wsum(z) + P[kPropOb3];
+        if (lane == rr + i) {
+          if (base == 0)
+            out.lg0 = z;
+          else
+            out.lg1 = z;
+        }
       }
     }
   }
-  *out0 = lg0;
-  *out1 = lg1;
+  return out;
 }
 
 // Softmax probability of row `target_row` among rows [r0, r1) whose logits sit in lanes.
 template <typename T>
-__device__ T warp_softmax_prob(T lg0, T lg1, int r0, int r1, int target_row) {
+__device__ __noinline__ T warp_softmax_prob(T lg0, T lg1, int r0, int r1, int target_row) {
   const int lane = threadIdx.x & 31;
   T zmax = -(T)INFINITY;
   for (int r = r0; r < r1; ++r) {
@@ -267,7 +307,7 @@ __device__ T warp_softmax_prob(T lg0, T lg1, int r0, int r1, int target_row) {
 
 // Appends the antiparallel neighbours of i (in CSR order) as rows (i -> u, x); all lanes
 // write the same values (warp-uniform), returns the new count.
-__device__ int push_rows(const DevGraph& g, const int8_t* sp, int i, int x, int pa, int pb, int* rc, int* ro, int* rx,
+__device__ __noinline__ int push_rows(const DevGraph& g, const int8_t* sp, int i, int x, int pa, int pb, int* rc, int* ro, int* rx,
                          int n) {
   const int a = x ? pa : -1, b = x ? pb : -1;
   const int si = spin_x(sp, i, a, b);
@@ -284,9 +324,112 @@ __device__ int push_rows(const DevGraph& g, const int8_t* sp, int i, int x, int 
   return n;
 }
 
-template <typename T>
+// Elements of the block's parameters: W (not with r8), its transpose, biases, embedding, readout.
+__host__ __device__ inline size_t metro_param_elems(int F, bool r8) {
+  const size_t n = (r8 ? 0 : (size_t)2 * F * (F + 1)) + (size_t)F * (2 * F + 4) + F + 2 * F + (F + 2) * 2 + 2;
+  return (n + 3) / 4 * 4;
+}
+__host__ __device__ inline int metro_meta_ints(int rows, int span) { return (3 * rows + span + 5) / 4 * 4; }
+
+// One layer of a proposal for one column a lane: rows [0, R) in groups of 8.  xs [2F][8]: the group's
+// dX = [A_hat dH ; dH], feature k of rows 0..3 and 4..7 as two 16-byte halves that swap places
+// every four k (the lanes' stores then spread over the banks).  Positions outside ball_{l-1} read the row of
+// zeros behind it.  pre: the lane's part of Re Delta at the last layer.
+__device__ __forceinline__ void metro_rows8(float* xs, const float* wt, const float* swr, const float* dprev,
+                                            float* dcur, float* dyl, const float* Y, const int* mv, const int* mdeg,
+                                            const int* mnb, const int2* nbw, int F, int R, int sprev, bool last,
+                                            float& pre) {
+  const int lane = threadIdx.x & 31;
+  const bool has = lane < F;
+  const int f = has ? lane : 0;
+  for (int rb = 0; rb < R; rb += 8) {
+    float yc[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) yc[q] = Y[(size_t)mv[min(rb + q, R - 1)] * F + f];
+    // two rows a turn: unrolled over all eight, this loop and the last one did not stay in the
+    // instruction caches (with 14 warps at different places of the step)
+#pragma unroll 1
+    for (int p = 0; p < 4; ++p) {
+      float ag[2], sf[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = min(rb + 2 * p + h, R - 1);
+        const int2* nb = nbw + mnb[r];
+        const int dg = mdeg[r];
+        float s = 0.f;
+#pragma unroll 1
+        for (int t = 0; t < dg; ++t) {
+          const int2 n = nb[t];
+          s = fmaf(__int_as_float(n.y), dprev[min(n.x, sprev) * F + f], s);
+        }
+        ag[h] = s;
+        sf[h] = dprev[min(r, sprev) * F + f];
+      }
+      if (has) {
+        float2* x = reinterpret_cast<float2*>(xs);
+        const int half = p >> 1;
+        x[4 * lane + 2 * (half ^ ((lane >> 2) & 1)) + (p & 1)] = make_float2(ag[0], ag[1]);
+        x[4 * (F + lane) + 2 * (half ^ (((F + lane) >> 2) & 1)) + (p & 1)] = make_float2(sf[0], sf[1]);
+      }
+    }
+    __syncwarp();
+    uint64_t acc[4] = {0, 0, 0, 0};
+    const ulonglong2* x2 = reinterpret_cast<const ulonglong2*>(xs);
+#pragma unroll 1
+    for (int k = 0; k < 2 * F; k += 8) {
+      float w[8];
+      load4(wt + k, w);
+      load4(wt + k + 4, w + 4);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint64_t w2 = f2_dup(w[u]);
+        const ulonglong2 a = x2[2 * (k + u) + (u >> 2)], b = x2[2 * (k + u) + ((u >> 2) ^ 1)];
+        acc[0] = f2_fma(a.x, w2, acc[0]);
+        acc[1] = f2_fma(a.y, w2, acc[1]);
+        acc[2] = f2_fma(b.x, w2, acc[2]);
+        acc[3] = f2_fma(b.y, w2, acc[3]);
+      }
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int r = rb; r < R && r < rb + 8; r += 2) {
+      float ys[2];
+      f2_unpack(acc[0], ys[0], ys[1]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        if (!has || r + h >= R) break;
+        const float d = dtanh(yc[h], ys[h]);
+        dyl[(size_t)(r + h) * F + lane] = ys[h];
+        if (last)
+          pre += d * swr[2 * lane];
+        else
+          dcur[(size_t)(r + h) * F + lane] = d;
+      }
+#pragma unroll
+      for (int i = 0; i < 3; ++i) acc[i] = acc[i + 1];
+#pragma unroll
+      for (int i = 0; i < 6; ++i) yc[i] = yc[i + 2];
+    }
+  }
+}
+
+// log(a) - log(b)
+__device__ __noinline__ double m_log_ratio(double a, double b) { return log(a) - log(b); }
+
+// PROP: learned moves.  NF: feature columns of a lane (F <= 32 NF).  For one column of float32
+// with F a multiple of 4 the layers take 8 rows at a time in packed multiply-adds (R8).
+//
+// What bounds it: instructions (some 30000 a learned step on a random graph of 65 sites, L 3, F 32) and
+// their supply -- every warp is at another place of a step that was longer than the instruction
+// caches (6 of 11 stall cycles an instruction).  So the learned and the plain kernel are apart,
+// one-column code is not carried through two, rare and repeated pieces are calls, loops over a
+// group's rows are rolled, and four rows of the network share the loads of its weights.  One sweep of
+// 4096 chains with learned moves: 37.6 -> 21.7 ms; plain FP32 sweep of 4096 chains on Kagome 108,
+// L 4, F 32: 18.2 -> 12.1; the two-column kernel gains from the calls alone (F 64, learned 10.4 -> 6.4).
+template <typename T, bool PROP, int NF>
 __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
+  constexpr bool R8 = sizeof(T) == 4 && NF == 1;
   const DevGraph& g = a.g;
   const Dims& m = a.m;
   const int N = m.N, F = m.F, L = m.L, E = m.E;
@@ -294,16 +437,15 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
   const int ldw = F + 1;
   // block-shared parameters: W (2F x F) and its transpose Wt (F x (2F + 4)) for 128-bit row loads
   const int ldt = 2 * F + 4;
-  T* sW = (T*)smem;                  // [2F][F+1]
-  T* sWt = sW + 2 * F * ldw;         // [F][2F+4]
+  T* sW = (T*)smem;                  // [2F][F+1], not with R8
+  T* sWt = sW + (R8 ? 0 : 2 * F * ldw);         // [F][2F+4]
   T* sb = sWt + F * ldt;             // [F]
   T* semb = sb + F;                  // [2][F]
   T* swr = semb + 2 * F;             // [(F+2)][2]
   T* sbr = swr + (F + 2) * 2;        // [2]
-  const size_t param_elems = (size_t)2 * F * ldw + (size_t)F * ldt + F + 2 * F + (F + 2) * 2 + 2;
-  const size_t param_pad = (param_elems + 3) / 4 * 4;
+  const size_t param_pad = metro_param_elems(F, R8);
   T* sP = (T*)smem + param_pad;  // proposal network (when used)
-  const size_t prop_pad = a.prop ? ((size_t)kPropParams + 3) / 4 * 4 : 0;
+  const size_t prop_pad = PROP ? ((size_t)kPropParams + 3) / 4 * 4 : 0;
   T* wbase = sP + prop_pad;
   unsigned char* wb = (unsigned char*)wbase + (size_t)warp * a.warp_bytes;
   T* wsm = (T*)wb;                                   // this warp's dH rows and staged dX rows
@@ -312,21 +454,22 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
   int* mdeg = mv + a.max_rows;                       // its degree
   int* mnb = mdeg + a.max_rows;                      // offset of its neighbour entries
   int* npos = mnb + a.max_rows;                      // per neighbour entry: position in the ball
-  T* nwt = (T*)(mv + ((3 * a.max_rows + a.max_span + 3) / 4 * 4));  // ... and normalised weight
+  T* nwt = (T*)(mv + metro_meta_ints(a.max_rows, a.max_span));  // ... and normalised weight
+  int2* nbw = (int2*)(mv + (3 * a.max_rows + 1) / 2 * 2);  // R8: both (position, weight bits)
   int* prc = (int*)(nwt + a.max_span);               // proposal rows: centre, partner, exchanged
   int* pro = prc + a.prop_rows;
   int* prx = pro + a.prop_rows;
   int8_t* spin = (int8_t*)(prx + a.prop_rows);
   const T* th = a.theta;
   for (int i = threadIdx.x; i < 2 * F * F; i += blockDim.x) {
-    sW[(i / F) * ldw + i % F] = th[m.oW + i];
+    if (!R8) sW[(i / F) * ldw + i % F] = th[m.oW + i];
     sWt[(i % F) * ldt + i / F] = th[m.oW + i];
   }
   for (int i = threadIdx.x; i < F; i += blockDim.x) sb[i] = th[m.ob + i];
   for (int i = threadIdx.x; i < 2 * F; i += blockDim.x) semb[i] = m_tanh(th[m.oWe + i] + th[m.obe + i % F]);
   for (int i = threadIdx.x; i < (F + 2) * 2; i += blockDim.x) swr[i] = th[m.owr + i];
   if (threadIdx.x < 2) sbr[threadIdx.x] = th[m.obr + threadIdx.x];
-  if (a.prop)
+  if (PROP)
     for (int i = threadIdx.x; i < kPropParams; i += blockDim.x) sP[i] = (T)a.prop[i];
   __syncthreads();
 
@@ -337,7 +480,7 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
   T* Hs1 = Hs0 + (size_t)N * F;
   T* dYg = Ybase;  // dY^l rows at dYg + off_dy[l]
   const int f0 = lane, f1 = lane + 32;
-  const bool has0 = f0 < F, has1 = f1 < F;
+  const bool has0 = f0 < F, has1 = NF > 1 && f1 < F;
   const int64_t n_steps = (int64_t)a.n_sweeps * N;
   const int n_rec = a.record_every > 0 ? a.n_sweeps / a.record_every : 0;
 
@@ -366,6 +509,20 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
         }
         const T sf0 = has0 ? Hp[(size_t)v * F + f0] : (T)0, sf1 = has1 ? Hp[(size_t)v * F + f1] : (T)0;
         T y0 = has0 ? sb[f0] : (T)0, y1 = has1 ? sb[f1] : (T)0;
+        if (R8) {
+          const T* wt = sWt + (size_t)(has0 ? f0 : 0) * ldt;
+          for (int k4 = 0; k4 < F; k4 += 4) {
+            T wa[4], wb[4];
+            load4(wt + k4, wa);
+            load4(wt + F + k4, wb);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              const T av = __shfl_sync(0xffffffffu, ag0, k4 + u);
+              const T sv = __shfl_sync(0xffffffffu, sf0, k4 + u);
+              y0 += av * wa[u] + sv * wb[u];
+            }
+          }
+        } else
         for (int kk = 0; kk < F; ++kk) {
           const T av = __shfl_sync(0xffffffffu, kk < 32 ? ag0 : ag1, kk & 31);
           const T sv = __shfl_sync(0xffffffffu, kk < 32 ? sf0 : sf1, kk & 31);
@@ -398,7 +555,7 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
       int e = -1, kind = 1;
       bool move = false;
       T logq = 0;
-      if (!a.prop) {
+      if (!PROP) {
         e = (int)__umul64hi(r0, (uint64_t)E);
         move = spin[__ldg(g.edges + 2 * e)] != spin[__ldg(g.edges + 2 * e + 1)];
       } else {
@@ -420,7 +577,9 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
           __syncwarp();
           if (n1 > 0) {
             // the partner j ~ pi_i(. | s), by the categorical uniform (r3 mod 2^32) 2^-32
-            warp_logits<T>(g, spin, sP, prc, pro, prx, n1, -1, -1, &lg0, &lg1);
+            const Logits<T> lg = warp_logits<T>(g, spin, sP, prc, pro, prx, n1, -1, -1);
+            lg0 = lg.lg0;
+            lg1 = lg.lg1;
             T zmax = -(T)INFINITY;
             for (int r = 0; r < n1; ++r) {
               const T z = __shfl_sync(0xffffffffu, r < 32 ? lg0 : lg1, r & 31);
@@ -458,13 +617,15 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
           const int g2 = n;
           n = push_rows(g, spin, pj, 1, pi, pj, prc, pro, prx, n);
           __syncwarp();
-          warp_logits<T>(g, spin, sP, prc, pro, prx, n, pi, pj, &lg0, &lg1);
+          const Logits<T> lg = warp_logits<T>(g, spin, sP, prc, pro, prx, n, pi, pj);
+          lg0 = lg.lg0;
+          lg1 = lg.lg1;
           const T p_ij = kind == 1 ? warp_softmax_prob<T>(lg0, lg1, 0, g0, row_of(pro, 0, g0, pj)) : pij;
           const T p_ji = warp_softmax_prob<T>(lg0, lg1, g0, g1, row_of(pro, g0, g1, pi));
           const T p_ij2 = warp_softmax_prob<T>(lg0, lg1, g1, g2, row_of(pro, g1, g2, pj));
           const T p_ji2 = warp_softmax_prob<T>(lg0, lg1, g2, n, row_of(pro, g2, n, pi));
           const T wl = ((T)1 - eps) / (T)N, wp = eps / (T)E;
-          logq = (T)(log((double)(wl * (p_ij2 + p_ji2) + wp)) - log((double)(wl * (p_ij + p_ji) + wp)));
+          logq = (T)m_log_ratio((double)(wl * (p_ij2 + p_ji2) + wp), (double)(wl * (p_ij + p_ji) + wp));
         }
       }
       double* tr = a.trace ? a.trace + ((size_t)ch * n_steps + k) * 4 : nullptr;
@@ -491,6 +652,7 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
             d0[f1] = semb[cj * F + f1] - semb[ci * F + f1];
             d0[F + f1] = semb[ci * F + f1] - semb[cj * F + f1];
           }
+          if (R8 && has0) d0[2 * F + f0] = 0;
           __syncwarp();
         }
         // row metadata of ball_L(e): vertex, degree, neighbour positions and weights
@@ -504,18 +666,29 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
           mdeg[r] = dg;
           mnb[r] = o;
           for (int t = 0; t < dg; ++t) {
-            npos[o + t] = __ldg(g.nbr_pos + nb_base + o + t);
-            nwt[o + t] = (T)__ldg(g.wd + k0 + t);
+            const int p = __ldg(g.nbr_pos + nb_base + o + t);
+            const T w = (T)__ldg(g.wd + k0 + t);
+            if (R8) {
+              nbw[o + t] = make_int2(p, __float_as_int((float)w));
+            } else {
+              npos[o + t] = p;
+              nwt[o + t] = w;
+            }
           }
         }
         __syncwarp();
-        T pre = 0, pim = 0;
+        T pre = 0;
         for (int l = 1; l <= L; ++l) {
           const int sprev = __ldg(bsz + l - 1), R = __ldg(bsz + l);
           const T* dprev = wsm + a.off_dh[l - 1];
           T* dcur = l < L ? wsm + a.off_dh[l] : nullptr;
           T* dyl = dYg + a.off_dy[l];
           const T* Y = Ybase + (size_t)(l - 1) * N * F;
+          if constexpr (R8) {
+            if (l < L && has0) dcur[(size_t)R * F + f0] = 0;
+            metro_rows8(sX, sWt + (size_t)(has0 ? f0 : 0) * ldt, swr, dprev, dcur, dyl, Y, mv, mdeg, mnb, nbw, F, R,
+                        sprev, l == L, pre);
+          } else
           for (int rb = 0; rb < R; rb += 4) {
             // stage dX = [A_hat dH^{l-1} ; dH^{l-1}] of rows rb..rb+3 (zeros past R)
 #pragma unroll
@@ -596,31 +769,25 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
                 dyl[(size_t)r * F + f0] = ys0[q];
                 if (l < L)
                   dcur[(size_t)r * F + f0] = d;
-                else {
+                else
                   pre += d * swr[2 * f0];
-                  pim += d * swr[2 * f0 + 1];
-                }
               }
               if (has1) {
                 const T d = dtanh(yc1[q], ys1[q]);
                 dyl[(size_t)r * F + f1] = ys1[q];
                 if (l < L)
                   dcur[(size_t)r * F + f1] = d;
-                else {
+                else
                   pre += d * swr[2 * f1];
-                  pim += d * swr[2 * f1 + 1];
-                }
               }
             }
           }
           __syncwarp();
         }
         const T dre = wsum(pre);
-        const T dim = wsum(pim);
-        (void)dim;
         T value;
         bool acc;
-        if (a.prop) {
+        if (PROP) {
           value = (T)2 * dre + logq;
           acc = m_accept_log<T>(r1, value);
         } else {
@@ -639,10 +806,23 @@ __global__ void __launch_bounds__(32 * kMetroMaxWarps) k_metro_warp(const MetroA
             const int R = __ldg(bsz + l);
             const T* dy = dYg + a.off_dy[l];
             T* Y = Ybase + (size_t)(l - 1) * N * F;
-            for (int r = 0; r < R; ++r) {
-              const int v = mv[r];
-              if (has0) Y[(size_t)v * F + f0] += dy[(size_t)r * F + f0];
-              if (has1) Y[(size_t)v * F + f1] += dy[(size_t)r * F + f1];
+            // four rows' loads before their stores (a ball's vertices are distinct)
+            for (int r = 0; r < R; r += 4) {
+              T y0[4], y1[4];
+              int v[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int rr = r + q < R ? r + q : R - 1;
+                v[q] = mv[rr];
+                y0[q] = has0 ? Y[(size_t)v[q] * F + f0] + dy[(size_t)rr * F + f0] : (T)0;
+                y1[q] = has1 ? Y[(size_t)v[q] * F + f1] + dy[(size_t)rr * F + f1] : (T)0;
+              }
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                if (r + q >= R) break;
+                if (has0) Y[(size_t)v[q] * F + f0] = y0[q];
+                if (has1) Y[(size_t)v[q] * F + f1] = y1[q];
+              }
             }
           }
           if (lane == 0) {
@@ -707,29 +887,42 @@ struct MetroPlan {
   size_t ws_bytes = 0;
 };
 
+// Columns a lane: one (with the packed rows) for F <= 32 and a multiple of 4.
+static int metro_nf(int F) { return F <= 32 && F % 4 == 0 ? 1 : 2; }
+
+template <typename T>
+static const void* metro_kernel(int F, bool prop) {
+  if (metro_nf(F) == 1)
+    return prop ? (const void*)k_metro_warp<T, true, 1> : (const void*)k_metro_warp<T, false, 1>;
+  return prop ? (const void*)k_metro_warp<T, true, 2> : (const void*)k_metro_warp<T, false, 2>;
+}
+
 template <typename T>
 static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int with_prop, MetroPlan* p) {
-  if (m.L < 1 || m.F > 64) return GNA_ERR_UNSUPPORTED;
+  // dX and W^T rows are read 4 features at a time, which needs 2F to be a multiple of 4
+  if (m.L < 1 || m.F > 64 || m.F % 2 != 0) return GNA_ERR_UNSUPPORTED;
   if (with_prop && g->max_deg > 16) return GNA_ERR_UNSUPPORTED;
   p->prop_rows = with_prop ? 4 * (g->max_deg > 0 ? g->max_deg : 1) : 0;
   DeviceInfo di;
   gna_status st = device_info(&di);
   if (st != GNA_OK) return st;
   const int F = m.F, L = m.L;
+  const bool r8 = sizeof(T) == 4 && metro_nf(F) == 1;
   // per-warp shared memory: dH rows (l < L), 4 staged dX rows, row metadata, spins
   int o = 0;
   for (int l = 0; l < L; ++l) {
     p->off_dh[l] = o;
-    o += g->max_ball[l] * F;
+    o += (g->max_ball[l] + (r8 ? 1 : 0)) * F;  // r8: and a row of zeros
   }
+  o = (o + 3) / 4 * 4;
   p->off_x = o;
-  o += 4 * 2 * F;
+  o += (r8 ? 8 : 4) * 2 * F;
   size_t bytes = (size_t)o * sizeof(T);
   bytes = (bytes + 15) / 16 * 16;
   p->off_meta = (int)bytes;
   p->max_rows = g->max_ball[L];
   p->max_span = g->max_span[L];
-  const int meta_ints = (3 * p->max_rows + p->max_span + 3) / 4 * 4;  // keeps the weights 16-byte aligned
+  const int meta_ints = metro_meta_ints(p->max_rows, p->max_span);  // keeps the weights 16-byte aligned
   bytes += (size_t)meta_ints * 4 + (size_t)p->max_span * sizeof(T) + (size_t)3 * p->prop_rows * 4 + (size_t)m.N;
   p->warp_bytes = (int)((bytes + 15) / 16 * 16);
   // per-warp workspace slot: Y^1..Y^L, two H scratch layers, dY^1..dY^L rows
@@ -739,17 +932,20 @@ static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int w
     e += (size_t)g->max_ball[l] * F;
   }
   p->ws_elems = (e + 31) / 32 * 32;
-  const size_t param_elems = (size_t)2 * F * (F + 1) + (size_t)F * (2 * F + 4) + F + 2 * F + (F + 2) * 2 + 2;
-  const size_t param_bytes = ((param_elems + 3) / 4 * 4 + (with_prop ? ((size_t)kPropParams + 3) / 4 * 4 : 0)) * sizeof(T);
+  const size_t param_bytes = (metro_param_elems(F, r8) + (with_prop ? ((size_t)kPropParams + 3) / 4 * 4 : 0)) * sizeof(T);
   auto smem_for = [&](int nw) { return param_bytes + (size_t)nw * p->warp_bytes; };
   int nw = kMetroMaxWarps;
   while (nw > 0 && smem_for(nw) > (size_t)di.smem_optin - 1024) --nw;
   if (nw < 2) return GNA_ERR_UNSUPPORTED;
+  // equal shares: the rounds over the chains that the most warps need, with as few warps as do them
+  const int64_t per_sm = (C + di.sms - 1) / di.sms, rounds = (per_sm + nw - 1) / nw;
+  nw = (int)((per_sm + rounds - 1) / rounds);
   p->nwarps = nw;
   p->smem = (int)smem_for(nw);
-  GNA_CUDA_TRY(cudaFuncSetAttribute((const void*)k_metro_warp<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
+  const void* kern = metro_kernel<T>(F, with_prop != 0);
+  GNA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
   int occ = 0;
-  GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k_metro_warp<T>, 32 * nw, p->smem));
+  GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * nw, p->smem));
   if (occ < 1) occ = 1;
   int64_t grid = (int64_t)di.sms * occ;
   const int64_t need = (C + nw - 1) / nw;
@@ -809,7 +1005,9 @@ static gna_status metro_launch_t(const MetroCall& mc, void* ws, size_t ws_bytes,
   a.trace = mc.trace;
   a.gws = (T*)ws;
   a.ws_elems = p.ws_elems;
-  k_metro_warp<T><<<p.grid, 32 * p.nwarps, p.smem, stream>>>(a);
+  void* args[] = {&a};
+  GNA_CUDA_TRY(cudaLaunchKernel(metro_kernel<T>(mc.m.F, mc.prop != nullptr), dim3(p.grid), dim3(32 * p.nwarps), args,
+                                p.smem, stream));
   GNA_CUDA_TRY(cudaGetLastError());
   return GNA_OK;
 }

@@ -179,6 +179,42 @@ def test_proposal_gradient(torch, name, n, n_up):
     np.testing.assert_allclose(grad.cpu().numpy(), want, rtol=0, atol=1e-4 * np.abs(want).max())
 
 
+@pytest.mark.parametrize("name,F,L,C", [("kagome2", 5, 2, 3), ("kagome2", 10, 2, 40), ("er30", 20, 3, 5), ("isolated", 32, 2, 7),
+                                        ("complete9", 4, 1, 9), ("kagome3", 32, 3, 5), ("er30", 48, 2, 3)])
+def test_fp32_sampler(torch, name, F, L, C):
+    # Delta in FP32: 1e-4 of its size or of one (rounding 6e-8 of each of some thousand terms)
+    g = GRAPHS[name]()
+    th, s0, tr, final = _sweep(torch, g, F, L, gna.PREC_FP32, 0.3, C, 2)
+    props = _replay(g, s0, tr, final, 31, 77, "fp32")
+    got, want = _deltas(th, F, L, g, props, 20)
+    assert np.abs(got - want).max() <= 1e-4 * max(1.0, np.abs(want).max())
+
+
+@pytest.mark.parametrize("name,F,L", [("er30", 32, 3), ("er30", 20, 2), ("complete9", 16, 2), ("kagome3", 48, 2), ("kagome2", 5, 2)])
+def test_fp32_learned_moves_as_fp64(torch, name, F, L):
+    # the first step of 400 chains: the same bond and kind as the FP64 sampler's (checked against the
+    # oracle elsewhere), the log acceptance ratio within 1e-4 of its size or of one; a chain may
+    # pick another partner where its uniform lies within 1e-6 of a probability (at most 2 of 400)
+    g = GRAPHS[name]()
+    th32 = torch.tensor(W.random_theta(F, L, seed=7, scale=0.3), dtype=torch.float32, device="cuda")
+    p32 = torch.tensor(W.random_proposal_params(3, 0.5), dtype=torch.float32, device="cuda")
+    graph = gna.Graph.from_workload(g, L)
+    s0 = W.random_spins(g.n_sites, 400, seed=4)
+    tr = {}
+    for prec, th in ((gna.PREC_FP32, th32), (gna.PREC_FP64, th32.double())):
+        ch = torch.tensor(s0, device="cuda")
+        tr[prec] = gna.metropolis_sweep(graph, gna.Model(F, L, prec), th, ch, 1, 0, 31, 0, trace=True, proposal=p32)[3].cpu().numpy()[:, 0]
+        x = ch.cpu().numpy()
+        assert np.array_equal((x > 0).sum(axis=1), (s0 > 0).sum(axis=1))
+    a, b = tr[gna.PREC_FP32], tr[gna.PREC_FP64]
+    same = a[:, 0] == b[:, 0]
+    assert same.sum() >= 398 and np.array_equal(a[:, 3], b[:, 3])
+    assert np.array_equal(np.isnan(a[same, 2]), np.isnan(b[same, 2]))
+    ok = same & ~np.isnan(b[:, 2])
+    assert ok.sum() > 100
+    assert (np.abs(a[ok, 2] - b[ok, 2]) <= 1e-4 * np.maximum(1.0, np.abs(b[ok, 2]))).all()
+
+
 @pytest.mark.parametrize("name,F,L,n", [("two", 16, 1, 1), ("isolated", 64, 3, 5), ("ring40", 48, 2, 153), ("kagome6", 32, 4, 1),
                                         ("kagome6", 64, 2, 700), ("tri14", 64, 2, 400), ("bipartite", 16, 3, 17)])
 def test_bf16x2_forward(torch, name, F, L, n):
