@@ -408,7 +408,7 @@ def measure_workload(key, prec_name, dev, flush, K_timed, peaks, peak_kind):
                                      "backward_sgd": float(ph[:, 2].mean())},
             "eloc_samples_per_s": Bn / (t_eloc / 1000.0),
             "sample_updates_per_s": Bn / (upd / 1000.0),
-            "roofline": {"bound": "tensor", "kernel": "%s (gna_local_energy_logpsi, %s)" % ("k_eloc" if prec == gna.PREC_BF16X2 else "k_tc", prec_name),
+            "roofline": {"bound": "tensor", "kernel": "%s (gna_local_energy_logpsi, %s)" % ("k_eloc" if prec_name == "bf16x2" else "k_tc", prec_name),
                          "achieved": achieved, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                          "frac": achieved / peaks["bf16_tflops_sustained"],
                          "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl,
