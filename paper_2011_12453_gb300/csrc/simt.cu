@@ -976,10 +976,12 @@ __global__ void __launch_bounds__(kThreads) k_metropolis(const SimtArgs<T> a) {
 }
 
 // Reverse mode of Eq. (gcn) and the readout; activations recomputed per sample.  512 threads an
-// SM (128 registers each), as four blocks of 128, two of 256 or one of 512 threads, the smallest
-// whose features fit shared memory: the phases of a small sample occupy few threads (2F F / 4 of
-// them in dW), and other samples' blocks fill in.  FP64 Kagome 2x2x3, F 16, 1024 samples: 245 us with
-// one block an SM.
+// SM (128 registers each), as four blocks of 128, two of 256 or one of 512 threads.  The phases of
+// a small sample occupy few threads (2F F / 4 of them in dW), and other samples' blocks fill in:
+// update of 1024 configurations, F 16, FP64 Kagome 2x2x3 0.81 -> 0.71 ms with four blocks, FP32 bosons on
+// 108 sites 1.28 -> 1.13.  One block where F F / 2 threads find work in it, where the features are in
+// the workspace (a drawn FP32 gradient took 12 % longer with four), and where the last round of
+// samples would leave more of the smaller blocks idle than they gain (a fifth).
 constexpr int kThreadsBwd = 512;
 
 template <typename T>
@@ -1231,8 +1233,11 @@ gna_status simt_plan(const gna_graph* g, const Dims& m, int op, int64_t B, Plan*
   }
   p->threads = kThreads;
   if (op == OP_BWD) {
-    int blocks = 4;
-    while (blocks > 1 && (size_t)blocks * (p->smem + 2048) > (size_t)di.smem_optin) blocks /= 2;
+    int blocks = p->region_in_smem ? 4 : 1;
+    auto rounds = [&](int k) { return (B + (int64_t)k * di.sms - 1) / ((int64_t)k * di.sms); };
+    while (blocks > 1 && ((size_t)blocks * (p->smem + 2048) > (size_t)di.smem_optin ||
+                          m.F * m.F / 2 > kThreadsBwd / blocks || 4 * blocks * rounds(blocks) > 5 * rounds(1)))
+      blocks /= 2;
     p->threads = kThreadsBwd / blocks;
   }
   const void* kp = kernel_ptr<T>(op);
