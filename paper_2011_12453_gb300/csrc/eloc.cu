@@ -138,7 +138,7 @@ static gna_status el_plan(const gna_graph* g, const Dims& m, int64_t B, bool f32
   int64_t grid = di.sms;
   if (grid > B) grid = B;
   p->grid = (int)(grid < 1 ? 1 : grid);
-  p->u_bytes = align_up((size_t)p->grid * (mode == EL_F32_LN ? 2 : 1) * m.L * m.N * el_ldu(m.F) * sizeof(float));
+  p->u_bytes = align_up((size_t)p->grid * 2 * m.L * m.N * el_ldu(m.F) * sizeof(float));
   p->ws_bytes = p->u_bytes + (p->a.h_smem ? 0 : align_up((size_t)p->grid * 2 * m.N * el_ldh(m.F) * sizeof(float)));
   return GNA_OK;
 }

@@ -21,8 +21,8 @@
 // tcgen05 every layer paid two block barriers and an MMA round trip (barrier 2.5 stalls per
 // instruction, 93 instructions per 32 features of a row).  One-warp units meet nobody.
 // Measured (local energy with log Psi, tensor-memory kernel before, this one after): Kagome
-// 108, L 4, F 32, 16384 configurations 33.9 -> 14.4 ms; triangular 144, L 4, F 48, 4001: 38.0 ->
-// 18.7 ms; Kagome 432, L 6, F 64, 512: 26.9 -> 18.2 ms; the error of the energies against 64 bits
+// 108, L 4, F 32, 16384 configurations 33.9 -> 14.7 ms; triangular 144, L 4, F 48, 4001: 38.0 ->
+// 18.4 ms; Kagome 432, L 6, F 64, 512: 26.9 -> 18.6 ms; the error of the energies against 64 bits
 // falls 3 to 5 times at weight scale 0.1.
 #pragma once
 
@@ -61,8 +61,8 @@ struct ElArgs {
   double* logpsi;
   double* eloc;
   float* dlogpsi;
-  float* gU;   // [grid][L][N][ldu] exp(2 Y) of the CTA's configuration (L2-resident), or with layer norm
-               // [grid][2][L][N][ldu] Y, then H
+  float* gU;   // [grid][2][L][N][ldu], L2-resident: exp(2 Y) of the CTA's configuration, then Y where that
+               // is out of range; with layer norm Y, then H
   float* gH;   // [grid][2][N][ldh] when the forward's rows are in the workspace
   int h_smem;
   int units, uw;                    // units per CTA, warps per unit
@@ -81,11 +81,25 @@ __device__ __forceinline__ void el_bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// What the incremental step needs of a cached unit, in one float32: E = exp(2 Y), at most
-// kElCap (Y = 43.7; zero below Y = -52).  H = (E - 1)/(E + 1), and 1 - H^2 = 4 E/(1 + E)^2 keeps its
-// relative precision at saturation.
-constexpr float kElCap = 5e37f;
-__device__ __forceinline__ float el_cache(float y) { return fminf(expf(2.f * y), kElCap); }
+// What the incremental step needs of a cached unit, in one float32: E = exp(2 Y).  H = (E - 1)/(E + 1),
+// and 1 - H^2 = 4 E/(1 + E)^2 keeps its relative precision at saturation.  Where E leaves
+// [kElTiny, kElCap) (Y outside -42.6 .. 43.4) it is 0 to kElTiny, kElCap or not a number, and Y itself
+// is kept beside the cache: a swing of more than 1 is then taken from Y (el_dtanh2_out), a smaller
+// one changes H by less than 1e-35.
+constexpr float kElCap = 5e37f, kElTiny = 1e-37f;
+__device__ __forceinline__ float el_cache(float y) {
+  const float e = expf(2.f * y);
+  return e > kElCap ? kElCap : e;  // (not fminf: what is not a number stays one)
+}
+__device__ __forceinline__ bool el_cached(float E) { return E >= kElTiny && E < kElCap; }
+// Four features' cache entries at U, and their Y at U + to_y where one of them needs it (true then).
+__device__ __forceinline__ bool el_store_cache(float* U, size_t to_y, float y0, float y1, float y2, float y3) {
+  const float4 e = make_float4(el_cache(y0), el_cache(y1), el_cache(y2), el_cache(y3));
+  *reinterpret_cast<float4*>(U) = e;
+  if (el_cached(e.x) && el_cached(e.y) && el_cached(e.z) && el_cached(e.w)) return false;
+  *reinterpret_cast<float4*>(U + to_y) = make_float4(y0, y1, y2, y3);
+  return true;
+}
 
 // The packed constants of el_dtanh2 and of the operand split.  Made by volatile assembly so
 // that they stay in registers: left to itself the compiler builds each of them anew, two
@@ -117,21 +131,36 @@ __device__ __forceinline__ uint64_t el_dtanh2(const ElConst& k, uint64_t x, uint
 }
 // The same for |x| > 1: with X = exp(-2 |x|), dH = 2 E/(1 + E) (1 - X)/(X + E) for x > 0 and
 // -2 E/(1 + E) (1 - X)/(1 + E X) for x < 0, in which nothing cancels or overflows, whichever way
-// the unit swings (one that lies outside the cached range stays where it is).
+// the unit swings (E within the cached range).
 __device__ __forceinline__ float el_dtanh_far(float x, float E) {
   const float X = expf(-2.f * fabsf(x));
   float r0, r1;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(1.f + E));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(x > 0.f ? fmaxf(X + E, 1e-37f) : fmaf(E, X, 1.f)));
-  return E < kElCap ? copysignf(2.f * (E * r0) * ((1.f - X) * r1), x) : 0.f;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(x > 0.f ? X + E : fmaf(E, X, 1.f)));
+  return copysignf(2.f * (E * r0) * ((1.f - X) * r1), x);
 }
-
 __device__ __forceinline__ uint64_t el_dtanh2_far(const ElConst& k, uint64_t x, uint64_t E) {
   float x0, x1, e0, e1, d0, d1;
   f2_unpack(el_dtanh2(k, x, E), d0, d1);
   f2_unpack(x, x0, x1);
   f2_unpack(E, e0, e1);
   return f2_pack(fabsf(x0) > 1.f ? el_dtanh_far(x0, e0) : d0, fabsf(x1) > 1.f ? el_dtanh_far(x1, e1) : d1);
+}
+// And outside the cached range, where tanh Y = sgn Y = +-1: dH = -2 sgn Y/(1 + exp(2 sgn Y (Y + x))).
+__device__ __forceinline__ float el_dtanh_out(float x, float y) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + expf(2.f * copysignf(1.f, y) * (y + x))));
+  return copysignf(2.f, -y) * r;
+}
+// el_dtanh2_far's d, put right where a unit of the pair is out of range (its Y at py).
+__device__ __forceinline__ uint64_t el_dtanh2_out(uint64_t d, uint64_t x, uint64_t E, const float* py) {
+  float x0, x1, e0, e1, d0, d1;
+  f2_unpack(d, d0, d1);
+  f2_unpack(x, x0, x1);
+  f2_unpack(E, e0, e1);
+  if (fabsf(x0) > 1.f && !el_cached(e0)) d0 = el_dtanh_out(x0, py[0]);
+  if (fabsf(x1) > 1.f && !el_cached(e1)) d1 = el_dtanh_out(x1, py[1]);
+  return f2_pack(d0, d1);
 }
 
 template <int FC>
@@ -145,9 +174,12 @@ struct ElCtx {
   const float* wf;
   const uint16_t* col;
   ElConst k;
+  // 1: some unit of the configuration is out of the cache's range (in shared memory; as a value it was
+  // a register of the whole tile and 7 % of a local energy on a random graph of 77 sites, F 32)
+  int* out;
 };
 
-// Forward of the configuration in c.spin: u of Y^1..Y^L into the cache, H^L left in the row
+// Forward of the configuration in c.spin: Y^1..Y^L into the cache, H^L left in the row
 // buffer that is returned when want_h.  X = [A_hat H ; H] as hi + lo operands, FP32 rows, in
 // the order of the forward call's kernel (bit-identical log Psi).
 template <int FC>
@@ -216,8 +248,8 @@ __device__ const float* el_forward_x2(const ElCtx<FC>& c, float* U, float* Hb, b
           if (v >= N) continue;
           const float y0 = D[0][2 * h] + bs.x, y1 = D[0][2 * h + 1] + bs.y;
           const float y2 = D[1][2 * h] + bs.z, y3 = D[1][2 * h + 1] + bs.w;
-          *reinterpret_cast<float4*>(U + ((size_t)(l - 1) * N + v) * LDU + 16 * co + 4 * q) =
-              make_float4(el_cache(y0), el_cache(y1), el_cache(y2), el_cache(y3));
+          float* u = U + ((size_t)(l - 1) * N + v) * LDU + 16 * co + 4 * q;
+          if (el_store_cache(u, (size_t)L * N * LDU, y0, y1, y2, y3)) *c.out = 1;
           if (l < L || want_h)
             *reinterpret_cast<float4*>(Hn + (size_t)v * LDH + 16 * co + 4 * q) =
                 make_float4(tanhf(y0), tanhf(y1), tanhf(y2), tanhf(y3));
@@ -370,10 +402,11 @@ __device__ void el_forward_f32(const ElCtx<FC>& c, float* U, float* Hb) {
           y[co][1] = D[2 * co][2 * h + 1] + bs.y;
           y[co][2] = D[2 * co + 1][2 * h] + bs.z;
           y[co][3] = D[2 * co + 1][2 * h + 1] + bs.w;
-          if (v < N)
-            *reinterpret_cast<float4*>(U + ((size_t)(l - 1) * N + v) * LDU + 16 * co + 4 * q) =
-                MODE == EL_F32_LN ? make_float4(y[co][0], y[co][1], y[co][2], y[co][3])
-                                  : make_float4(el_cache(y[co][0]), el_cache(y[co][1]), el_cache(y[co][2]), el_cache(y[co][3]));
+          float* u = U + ((size_t)(l - 1) * N + v) * LDU + 16 * co + 4 * q;
+          if (v < N && MODE == EL_F32_LN)
+            *reinterpret_cast<float4*>(u) = make_float4(y[co][0], y[co][1], y[co][2], y[co][3]);
+          else if (v < N && el_store_cache(u, (size_t)L * N * LDU, y[co][0], y[co][1], y[co][2], y[co][3]))
+            *c.out = 1;
         }
         if (MODE == EL_F32_LN) el_relu_ln<FC>(y);  // (shuffles: every lane)
         if (v < N)
@@ -429,7 +462,7 @@ __device__ __forceinline__ float el_max3(float a, float b, float c) {
 // One tile of 16 rows of a bond's ball_l: rows 16 t + g and + 8.
 //   zin: Z of the sp rows of ball_{l-1}, then a zero row, which stands for every row outside
 //   the ball; zout: Z of the n rows of ball_l for the next layer; Ul: the layer's cache (to_h
-//   floats on: its H, with layer norm).
+//   floats on: its H with layer norm, else Y of the units out of the cache's range).
 // The stages are kept apart (look-ups, gather, difference, product), each a block without
 // branches over all of the thread's values: a warp hides most of its own latency that way.
 template <int FC, int NP, int MODE, bool LAST>
@@ -531,8 +564,13 @@ __device__ __forceinline__ void el_tile(const ElCtx<FC>& c, uint32_t rec, uint32
 #pragma unroll
       for (int cc = 0; cc < FC; ++cc) {
         const ulonglong2 e = *reinterpret_cast<const ulonglong2*>(ur[h] + 16 * cc);
-        x[h][cc][0] = el_dtanh2_far(c.k, x[h][cc][0], e.x);
-        x[h][cc][1] = el_dtanh2_far(c.k, x[h][cc][1], e.y);
+        uint64_t d0 = el_dtanh2_far(c.k, x[h][cc][0], e.x), d1 = el_dtanh2_far(c.k, x[h][cc][1], e.y);
+        if (*c.out) {
+          d0 = el_dtanh2_out(d0, x[h][cc][0], e.x, ur[h] + to_h + 16 * cc);
+          d1 = el_dtanh2_out(d1, x[h][cc][1], e.y, ur[h] + to_h + 16 * cc + 2);
+        }
+        x[h][cc][0] = d0;
+        x[h][cc][1] = d1;
       }
   }
   const bool ok0 = row0 < n, ok1 = row0 + 8 < n;
@@ -623,7 +661,7 @@ __device__ __forceinline__ void el_tile(const ElCtx<FC>& c, uint32_t rec, uint32
 template <int FC, int NP, int MODE>
 __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ ElArgs a) {
   unsigned char* const smem = el_smem;
-  __shared__ int s_cnt[kElWarps];
+  __shared__ int s_cnt[kElWarps], s_out;
   __shared__ double s_diag[kElWarps], s_e[2 * kElWarps];
   constexpr int F = 16 * FC, LDH = el_ldh(F), LDU = el_ldu(F);
   const int N = a.m.N, L = a.m.L, E = a.m.E;
@@ -642,6 +680,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
   c.rp = (const int*)(smem + a.orp);
   c.wf = (const float*)(smem + a.owf);
   c.col = (const uint16_t*)(smem + a.ocol);
+  c.out = &s_out;
   c.k = {el_keep(63.f), el_keep(7.f), el_keep(1.f / 15.f), el_keep(28.f), el_keep(0.5f), el_keep(-1.f)};
   float* red = (float*)(smem + a.ored);
   const float* th = a.theta;
@@ -687,7 +726,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
     ((float*)c.z0)[i] = z;
   }
   const size_t to_h = (size_t)L * N * LDU;
-  float* U = a.gU + (size_t)blockIdx.x * to_h * (MODE == EL_F32_LN ? 2 : 1);
+  float* U = a.gU + (size_t)blockIdx.x * to_h * 2;
   float* Hb = a.h_smem ? (float*)(smem + a.oH) : a.gH + (size_t)blockIdx.x * 2 * N * LDH;
 
   // this thread's unit
@@ -713,6 +752,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
     }
     if (a.dlogpsi)
       for (int e = tid; e < E; e += kElThreads) a.dlogpsi[b * E + e] = 0.f;
+    if (tid == 0) s_out = 0;
     __syncthreads();
     const float* HL = nullptr;
     if (MODE == EL_X2)
