@@ -80,9 +80,13 @@ __device__ __forceinline__ double2 db_cache(double y) {
 // dH = tanh(Y + x) - tanh(Y) = t S/(1 + H t), t = tanh x, from H = tanh Y and S = 1 - H^2; NEXT also
 // the new H and S = S (1 - t^2)/(1 + H t)^2.  t = w/Q by a convergent of Lambert's continued
 // fraction: the sixth (relative error 4e-17 up to |x| = 1/4) or the ninth (3e-17 up to 1), chosen
-// for the whole warp.  Beyond 1 from X = exp(-2 |x|), with 1 + H t summed without cancellation.
+// for the whole warp.  Beyond 1 from X = exp(-2 |x|), with 1 + H t summed without cancellation; where S
+// is below kDbTiny (|Y| > 345; or not a number) it no longer says how far out the unit is, tanh Y = sgn Y
+// and dH = -2 sgn Y/(1 + exp(2 sgn Y (Y + x))), from Y at *py.
+constexpr double kDbTiny = 1e-300;
+__device__ __forceinline__ bool db_cached(double S) { return S >= kDbTiny; }
 template <bool NEXT>
-__device__ __forceinline__ double db_dtanh(double x, double2 hs, double2& next) {
+__device__ __forceinline__ double db_dtanh(double x, double2 hs, const double* py, double2& next) {
   const int hx = __double2hiint(x) & 0x7fffffff;
   const double z = x * x, H = hs.x, S = hs.y;
   double w, Q;
@@ -97,11 +101,19 @@ __device__ __forceinline__ double db_dtanh(double x, double2 hs, double2& next) 
   double d = w * u;
   if (NEXT) next = make_double2(H + d, (u * r) * ((Q - w) * (Q + w)));
   if (hx > 0x3ff00000) {  // (also what is not a number, which stays one)
-    const double X = exp(-2.0 * fabs(x)), x1 = 1.0 / (1.0 + X), t = copysign((1.0 - X) * x1, x), ah = fabs(H);
-    const double D = (x < 0.0) == (H < 0.0) ? 1.0 + ah * fabs(t) : S / (1.0 + ah) + ah * (2.0 * X * x1);
-    const double v = D > 0.0 ? S / D : 0.0;
-    d = t * v;
-    if (NEXT) next = make_double2(H + d, D > 0.0 ? v / D * (4.0 * X * (x1 * x1)) : S);
+    const bool in = db_cached(S);
+    const double y = in ? 0.0 : *py, sg = copysign(1.0, y);
+    const double X = exp(in ? -2.0 * fabs(x) : 2.0 * sg * (y + x)), x1 = 1.0 / (1.0 + X);
+    if (in) {
+      const double t = copysign((1.0 - X) * x1, x), ah = fabs(H);
+      const double D = (x < 0.0) == (H < 0.0) ? 1.0 + ah * fabs(t) : S / (1.0 + ah) + ah * (2.0 * X * x1);
+      const double v = S / D;  // (D is at least half of S)
+      d = t * v;
+      if (NEXT) next = make_double2(H + d, v / D * (4.0 * X * (x1 * x1)));
+    } else {
+      d = -2.0 * sg * x1;
+      if (NEXT) next = make_double2(sg * (X - 1.0) * x1, 4.0 * (X * x1) * x1);
+    }
     if (x != x) d = x;
   }
   return d;
@@ -160,9 +172,10 @@ __device__ __forceinline__ void db_rowmul(const double* x, const double* W, int 
   }
 }
 
-// Forward of spins sp by `nwarps` warps (this one is `warp`): Y (when Yc) and (H, 1 - H^2) of every
-// layer into the cache.  Hb: two row buffers [N][F]; xs: this warp's staging rows [rows_per_warp][2 F].
-template <int FPL, typename Sync>
+// Forward of spins sp by `nwarps` warps (this one is `warp`): (H, 1 - H^2) of every layer into the cache, and
+// Y (all of it with KEEP_Y, else of the units whose 1 - H^2 does not say how far out they are).  Hb: two row
+// buffers [N][F]; xs: this warp's staging rows [rows_per_warp][2 F].
+template <int FPL, bool KEEP_Y, typename Sync>
 __device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc, double2* Hc, double* Hb, double* xs,
                                     int warp, int nwarps, Sync sync) {
   const DbArgs& a = *c.a;
@@ -211,8 +224,8 @@ __device__ const double* db_forward(const DbCtx& c, const int8_t* sp, double* Yc
       for (int j = 0; j < FPL; ++j) {
         if (has[j] && v0 + c.row_in_warp < N) {
           const size_t i = ((size_t)(l - 1) * N + v) * F + fs[j];
-          if (Yc) Yc[i] = y[j];
           const double2 hs = db_cache(y[j]);
+          if (KEEP_Y || !db_cached(hs.y)) Yc[i] = y[j];
           Hc[i] = hs;
           Hn[(size_t)v * F + fs[j]] = hs.x;
         }
@@ -282,7 +295,7 @@ __device__ __forceinline__ void db_delta(const DbCtx& c, int info, const int8_t*
       for (int j = 0; j < FPL; ++j) {
         x[j] = fma(av, x[j], zi[min(r, prev) * 2 * F + F + fs[j]]);
         double2 nx;
-        dv[j] = db_dtanh<NEXT>(x[j], Hc[ci + fs[j]], nx);
+        dv[j] = db_dtanh<NEXT>(x[j], Hc[ci + fs[j]], Yc + ci + fs[j], nx);
         if (NEXT && ok && has[j]) {
           const double Yn = Yc[ci + fs[j]] + x[j];
           // far out, where 1 - H^2 nears the end of the exponents, from Y itself
@@ -354,7 +367,7 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
   for (int64_t ch = (int64_t)blockIdx.x * a.units + h; ch < a.B; ch += (int64_t)gridDim.x * a.units) {
     for (int v = utid; v < N; v += uthreads) sp[v] = a.chain_spins[ch * N + v];
     sync();
-    db_forward<FPL>(c, sp, Yc, Hc, wsu + a.off_h, (double*)(db_smem + uo + a.uz[0]) + (size_t)uwarp * c.rows_per_warp * 2 * F, uwarp,
+    db_forward<FPL, true>(c, sp, Yc, Hc, wsu + a.off_h, (double*)(db_smem + uo + a.uz[0]) + (size_t)uwarp * c.rows_per_warp * 2 * F, uwarp,
                     a.uw, sync);
     int accepts = 0;
     int64_t base = -32, k = 0, rec = 0;
@@ -505,12 +518,13 @@ __global__ void __launch_bounds__(kDbThreads) k_db_eloc(const __grid_constant__ 
   };
   double* wsu = a.ws + (size_t)blockIdx.x * a.ws_unit;
   double2* Hc = (double2*)wsu;
+  double* Yc = wsu + 2 * L * (size_t)N * F;
   for (int64_t b = blockIdx.x; b < a.B; b += gridDim.x) {
     for (int v = threadIdx.x; v < N; v += kDbThreads) sp[v] = a.spins[b * N + v];
     if (a.dlogpsi)
       for (int e = threadIdx.x; e < E; e += kDbThreads) a.dlogpsi[b * E + e] = 0.f;
     __syncthreads();
-    db_forward<FPL>(c, sp, nullptr, Hc, wsu + a.off_h,
+    db_forward<FPL, false>(c, sp, Yc, Hc, wsu + a.off_h,
                     (double*)(db_smem + a.ounit + (size_t)(a.units - 1) * a.unit_bytes + a.ud) + (size_t)warp * c.rows_per_warp * 2 * F,
                     warp, kDbWarps, [] { __syncthreads(); });
     // antiparallel bonds in order, and the diagonal energy
@@ -547,7 +561,7 @@ __global__ void __launch_bounds__(kDbThreads) k_db_eloc(const __grid_constant__ 
           const int e = list[b0 + i];
           const int info = __ldg(a.g.bond_info + (size_t)e * 32 + lane);
           double dre = 0.0, dim = 0.0;
-          db_delta<FPL, false, true>(c, info, sp, nullptr, Hc, nullptr, uo, uwarp, sync, dre, dim);
+          db_delta<FPL, false, true>(c, info, sp, Yc, Hc, nullptr, uo, uwarp, sync, dre, dim);
           dre = db_sum(dre);
           dim = db_sum(dim);
           if (a.uw > 1) {
@@ -698,7 +712,7 @@ gna_status db_plan(const gna_graph* g, const Dims& m, bool eloc, int64_t B, DbPl
   if (grid > need) grid = need;
   p->grid = (int)(grid < 1 ? 1 : grid);
   const size_t NF = (size_t)m.N * m.F;
-  size_t o = (eloc ? 2 : 3) * m.L * NF;  // (H, 1 - H^2), and Y in the sampler
+  size_t o = 3 * m.L * NF;  // (H, 1 - H^2), then Y
   if (!eloc)
     for (int l = 1; l <= m.L; ++l) {
       a.off_new[l] = o;

@@ -51,7 +51,8 @@ def _rounded(torch, th, F, prec):
     return theta, th
 
 
-@pytest.mark.parametrize("prec,A,b", [("fp32", 56.0, -5.0), ("fp32", 200.0, 60.0), ("bf16x2", 56.0, -5.0), ("bf16x2", 128.0, 60.0)])
+@pytest.mark.parametrize("prec,A,b", [("fp32", 56.0, -5.0), ("fp32", 200.0, 60.0), ("bf16x2", 56.0, -5.0), ("bf16x2", 128.0, 60.0),
+                                      ("fp64", 56.0, -5.0), ("fp64", 450.0, -20.0)])
 @pytest.mark.parametrize("F,L", [(16, 1), (32, 2)])
 def test_swings(torch, prec, A, b, F, L):
     g = W.kagome(3)
@@ -80,7 +81,7 @@ def test_swings(torch, prec, A, b, F, L):
         assert np.all(np.abs(dl - want_d) <= lim), np.max(np.abs(dl - want_d) - lim)
 
 
-@pytest.mark.parametrize("prec,A,b", [("fp32", 56.0, -5.0), ("bf16x2", 56.0, -5.0)])
+@pytest.mark.parametrize("prec,A,b", [("fp32", 56.0, -5.0), ("bf16x2", 56.0, -5.0), ("fp64", 450.0, -20.0)])
 def test_swings_in_the_samplers(torch, prec, A, b):
     # every proposal's Delta (the later ones start from rows that accepted moves have carried across)
     F, L = 16, 2
@@ -132,7 +133,7 @@ def test_fp32_local_energy_at_weight_scale_3(torch, F, L):
     assert np.all(np.abs(dl - want) <= lim), np.max(np.abs(dl - want) - lim)
 
 
-@pytest.mark.parametrize("prec", ["fp32", "bf16x2"])
+@pytest.mark.parametrize("prec", list(PREC))
 @pytest.mark.parametrize("name,scale", [("kagome2", 0.3), ("kagome2", 2.0), ("two", None)])
 def test_a_bias_that_is_not_a_number_shows_in_the_energy(torch, prec, name, scale):
     # "two": the only rows are the exchanged pair's, and the feature swings by more than 100
