@@ -133,7 +133,8 @@ GNA_API const char* gna_status_string(gna_status s);
  *   J         host float64 [n_edges]: coupling J_e of bond e (finite)
  *   max_layers 0..8: the largest L a model may use with this graph
  *   out       receives the handle (set to NULL on error)
- * Errors: GNA_ERR_INVALID_ARG (checked before any device call), GNA_ERR_CUDA. */
+ * Errors: GNA_ERR_INVALID_ARG (checked before any device call), GNA_ERR_CUDA,
+ * GNA_ERR_UNSUPPORTED when the host has no memory for the bonds' neighbourhood tables. */
 GNA_API gna_status gna_graph_create(int32_t n_sites, int32_t n_edges, const int32_t* edges,
                             const double* J, int32_t max_layers, gna_graph** out);
 

@@ -5,6 +5,8 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <utility>
 #include <vector>
 
@@ -128,13 +130,13 @@ void build(int n, int E, const int32_t* edges, const double* J, int Lmax, HostGr
       ents += d;
       npairs += (d + 1) / 2;
     }
-    if (e == 0) {  // room for bonds like the first one
-      const size_t R = (size_t)E * rows, N2 = (size_t)E * ents;
+    if (e == 0) {  // room for bonds like the first one, within reason: it may be a hub's, the others not
+      const size_t bonds = std::min((size_t)E, (size_t)(1 << 20) / (ents + rows) + 1), R = bonds * rows, N2 = bonds * ents;
       for (std::vector<int>* v : {&h->ball_vert, &h->row_nbr, &h->row_pack}) v->reserve(R);
       h->nbr_pos.reserve(N2);
       h->nbr_pos16.reserve(N2);
-      h->rec.reserve((size_t)E * ((rows + 1) / 2 * 4));
-      h->pairs.reserve((size_t)E * ((npairs + 3) / 4 * 4));
+      h->rec.reserve(bonds * ((rows + 1) / 2 * 4));
+      h->pairs.reserve(bonds * ((npairs + 3) / 4 * 4));
     }
     const size_t r0 = h->ball_vert.size(), e0 = h->nbr_pos.size();
     h->ball_off[e] = (int)r0;
@@ -247,7 +249,8 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
     if (hz) h.hz[e] = hz[e];
     if (cb) h.cb[e] = cb[e];
   }
-  gna_graph* g = new gna_graph();
+  std::unique_ptr<gna_graph, gna_status (*)(gna_graph*)> own(new gna_graph(), gna_graph_destroy);
+  gna_graph* const g = own.get();
   cudaGetDevice(&g->device);
   g->d.n = h.n;
   g->d.E = h.E;
@@ -276,10 +279,7 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
   pk.add(h.pairs, &g->d.pairs);
   pk.add(h.bond_info, &g->d.bond_info);
   st = pk.upload(g);
-  if (st != GNA_OK) {
-    gna_graph_destroy(g);
-    return st;
-  }
+  if (st != GNA_OK) return st;
   g->pack_ok = h.pack_ok;
   g->h_row_ptr = h.row_ptr;
   g->h_col = h.col;
@@ -295,8 +295,18 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
     g->max_deg = std::max(g->max_deg, h.row_ptr[v + 1] - h.row_ptr[v]);
     g->min_deg = std::min(g->min_deg, h.row_ptr[v + 1] - h.row_ptr[v]);
   }
-  *out = g;
+  *out = own.release();
   return GNA_OK;
+}
+
+// No exception leaves the C entries: the tables that the host has no memory for are refused.
+template <typename Fn>
+gna_status guarded(Fn fn) {
+  try {
+    return fn();
+  } catch (const std::exception&) {
+    return GNA_ERR_UNSUPPORTED;
+  }
 }
 
 }  // namespace
@@ -304,7 +314,7 @@ gna_status create_graph(int32_t n_sites, int32_t n_edges, const int32_t* edges, 
 
 extern "C" gna_status gna_graph_create(int32_t n_sites, int32_t n_edges, const int32_t* edges,
                                        const double* J, int32_t max_layers, gna_graph** out) {
-  return gna::create_graph(n_sites, n_edges, edges, J, J, nullptr, nullptr, max_layers, out);
+  return gna::guarded([&] { return gna::create_graph(n_sites, n_edges, edges, J, J, nullptr, nullptr, max_layers, out); });
 }
 
 extern "C" gna_status gna_graph_create_xxz(int32_t n_sites, int32_t n_edges, const int32_t* edges,
@@ -312,7 +322,7 @@ extern "C" gna_status gna_graph_create_xxz(int32_t n_sites, int32_t n_edges, con
                                            const double* c, int32_t max_layers, gna_graph** out) {
   if (n_edges > 0 && (Jz == nullptr || Jxy == nullptr || hz == nullptr || c == nullptr))
     return GNA_ERR_INVALID_ARG;
-  return gna::create_graph(n_sites, n_edges, edges, Jz, Jxy, hz, c, max_layers, out);
+  return gna::guarded([&] { return gna::create_graph(n_sites, n_edges, edges, Jz, Jxy, hz, c, max_layers, out); });
 }
 
 extern "C" gna_status gna_graph_destroy(gna_graph* g) {
@@ -339,10 +349,12 @@ extern "C" gna_status gna_ball_sizes_host(int32_t n_sites, int32_t n_edges, cons
                                           int32_t n_layers, int32_t* out) {
   using namespace gna;
   if (!out && n_edges > 0) return GNA_ERR_INVALID_ARG;
-  gna_status st = validate(n_sites, n_edges, edges, nullptr, n_layers, false);
-  if (st != GNA_OK) return st;
-  HostGraph h;
-  build(n_sites, n_edges, edges, nullptr, n_layers, &h);
-  std::memcpy(out, h.ball_size.data(), h.ball_size.size() * sizeof(int32_t));
-  return GNA_OK;
+  return guarded([&] {
+    gna_status st = validate(n_sites, n_edges, edges, nullptr, n_layers, false);
+    if (st != GNA_OK) return st;
+    HostGraph h;
+    build(n_sites, n_edges, edges, nullptr, n_layers, &h);
+    std::memcpy(out, h.ball_size.data(), h.ball_size.size() * sizeof(int32_t));
+    return (gna_status)GNA_OK;
+  });
 }
