@@ -901,6 +901,8 @@ template <typename T>
 static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int with_prop, MetroPlan* p) {
   // dX and W^T rows are read 4 features at a time, which needs 2F to be a multiple of 4
   if (m.L < 1 || m.F > 64 || m.F % 2 != 0) return GNA_ERR_UNSUPPORTED;
+  // one W in shared memory for every layer: models with a W per layer take the CTA-per-chain sampler
+  if (!m.shared && m.L > 1) return GNA_ERR_UNSUPPORTED;
   if (with_prop && g->max_deg > 16) return GNA_ERR_UNSUPPORTED;
   p->prop_rows = with_prop ? 4 * (g->max_deg > 0 ? g->max_deg : 1) : 0;
   DeviceInfo di;
