@@ -178,7 +178,8 @@ GNA_API gna_status gna_model_desc_init(gna_model_desc* d, int32_t F, int32_t L, 
 GNA_API int64_t gna_num_params(const gna_model_desc* d);
 
 /* Workspace bytes the call `op` needs for a batch of B configurations (B = number of
- * chains for GNA_OP_METROPOLIS) on the current device.  0 is a valid answer. */
+ * chains for GNA_OP_METROPOLIS) on the current device.  0 is a valid answer.  It never falls
+ * as B grows: a workspace for the largest batch does for all smaller ones. */
 GNA_API gna_status gna_workspace_size(const gna_graph* g, const gna_model_desc* d, int32_t op,
                               int64_t B, size_t* bytes);
 

@@ -940,6 +940,7 @@ static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int w
   while (nw > 0 && smem_for(nw) > (size_t)di.smem_optin - 1024) --nw;
   if (nw < 2) return GNA_ERR_UNSUPPORTED;
   // equal shares: the rounds over the chains that the most warps need, with as few warps as do them
+  const int most = nw;
   const int64_t per_sm = (C + di.sms - 1) / di.sms, rounds = (per_sm + nw - 1) / nw;
   nw = (int)((per_sm + rounds - 1) / rounds);
   p->nwarps = nw;
@@ -948,13 +949,19 @@ static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int w
   GNA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * nw, p->smem));
+  if (occ > kMetroMaxWarps / nw) occ = kMetroMaxWarps / nw;
   if (occ < 1) occ = 1;
   int64_t grid = (int64_t)di.sms * occ;
   const int64_t need = (C + nw - 1) / nw;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   p->grid = (int)grid;
-  p->ws_bytes = align_up((size_t)grid * nw * p->ws_elems * sizeof(T));
+  // The bytes of any number of chains up to C (fewer chains may be more warps): at most the warps that fit
+  // an SM's shared memory, kMetroMaxWarps of them, or the chains with a last block part empty.
+  int64_t slots = ((int64_t)di.smem_optin - (int64_t)param_bytes) / p->warp_bytes;
+  slots = di.sms * (slots < kMetroMaxWarps ? slots : kMetroMaxWarps);
+  if (slots > C + most - 1) slots = C + most - 1;
+  p->ws_bytes = align_up((size_t)slots * p->ws_elems * sizeof(T));
   return GNA_OK;
 }
 

@@ -630,6 +630,7 @@ gna_status mt_plan(const gna_graph* g, const Dims& m, int64_t C, MtPlan* p) {
   if (form == 3) return GNA_ERR_UNSUPPORTED;
   if (warps > mt_warps(m.F / 16)) warps = mt_warps(m.F / 16);
   // equal shares of the chains: the rounds that the most warps need, with as few warps as do them
+  const int most = warps;
   const int64_t per_sm = (C + di.sms - 1) / di.sms;
   const int64_t rounds = (per_sm + warps - 1) / warps;
   warps = (int)((per_sm + rounds - 1) / rounds);
@@ -638,7 +639,9 @@ gna_status mt_plan(const gna_graph* g, const Dims& m, int64_t C, MtPlan* p) {
   GNA_CUDA_TRY(cudaFuncSetAttribute(mt_kernel(m.F, form > 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
   const int64_t need = (C + warps - 1) / warps;
   p->grid = (int)(need < di.sms ? need : di.sms);
-  p->ws_bytes = align_up((size_t)p->grid * warps * a.ws_warp);
+  // (the bytes of any number of chains up to C: fewer chains may be more warps)
+  const int64_t slots = C + most - 1 < (int64_t)di.sms * most ? C + most - 1 : (int64_t)di.sms * most;
+  p->ws_bytes = align_up((size_t)slots * a.ws_warp);
   return GNA_OK;
 }
 

@@ -1232,12 +1232,14 @@ gna_status simt_plan(const gna_graph* g, const Dims& m, int op, int64_t B, Plan*
     p->smem = (int)out.total;
   }
   p->threads = kThreads;
+  int most = 0;  // blocks an SM of any batch (backward)
   if (op == OP_BWD) {
     int blocks = p->region_in_smem ? 4 : 1;
-    auto rounds = [&](int k) { return (B + (int64_t)k * di.sms - 1) / ((int64_t)k * di.sms); };
-    while (blocks > 1 && ((size_t)blocks * (p->smem + 2048) > (size_t)di.smem_optin ||
-                          m.F * m.F / 2 > kThreadsBwd / blocks || 4 * blocks * rounds(blocks) > 5 * rounds(1)))
+    while (blocks > 1 && ((size_t)blocks * (p->smem + 2048) > (size_t)di.smem_optin || m.F * m.F / 2 > kThreadsBwd / blocks))
       blocks /= 2;
+    most = blocks;
+    auto rounds = [&](int k) { return (B + (int64_t)k * di.sms - 1) / ((int64_t)k * di.sms); };
+    while (blocks > 1 && 4 * blocks * rounds(blocks) > 5 * rounds(1)) blocks /= 2;
     p->threads = kThreadsBwd / blocks;
   }
   const void* kp = kernel_ptr<T>(op);
@@ -1251,7 +1253,13 @@ gna_status simt_plan(const gna_graph* g, const Dims& m, int op, int64_t B, Plan*
   p->grid = (int)grid;
   size_t ws = 0;
   if (!p->region_in_smem) ws += align_up((size_t)p->grid * rel * sizeof(T));
-  if (part) ws += align_up((size_t)p->grid * m.P * sizeof(double));
+  if (part) {
+    // the bytes of any batch up to B: a smaller one may be more blocks
+    int64_t slots = (int64_t)di.sms * most;
+    if (slots > B) slots = B;
+    if (slots < grid) slots = grid;
+    ws += align_up((size_t)slots * m.P * sizeof(double));
+  }
   p->ws_bytes = ws;
   return GNA_OK;
 }
