@@ -121,6 +121,12 @@ struct DeviceInfo {
   int cc = 0;
 };
 gna_status device_info(DeviceInfo* out);
+// Lets a kernel take up to `limit` bytes of dynamic shared memory: the same limit for every plan of the
+// kernel (the device's, less its static variables), since host threads with other plans may be launching it.
+inline gna_status allow_smem(const void* kernel, uint64_t limit) {
+  GNA_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit));
+  return GNA_OK;
+}
 
 // Arguments of one SIMT launch (simt.cu).  op: 0 forward, 1 full local energy,
 // 2 incremental local energy, 3 Metropolis sweeps, 4 backward.

@@ -702,7 +702,7 @@ gna_status db_plan(const gna_graph* g, const Dims& m, bool eloc, int64_t B, DbPl
   if (uw > kDbWarps) return GNA_ERR_UNSUPPORTED;
   p->smem = (uint32_t)smem;
   const void* k = db_kernel(eloc, m.F);
-  GNA_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
+  if ((st = allow_smem(k, budget)) != GNA_OK) return st;
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kDbThreads, p->smem));
   if (occ < 1) occ = 1;

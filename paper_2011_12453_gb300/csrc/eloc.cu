@@ -134,7 +134,7 @@ static gna_status el_plan(const gna_graph* g, const Dims& m, int64_t B, bool f32
   p->smem = (uint32_t)el_layout(g, m, bu, bw, bn, mode, &p->a);
   const void* kfn = el_kernel(g, m.F, mode);
   p->kernel = kfn;
-  GNA_CUDA_TRY(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
+  if ((st = allow_smem(kfn, budget)) != GNA_OK) return st;
   int64_t grid = di.sms;
   if (grid > B) grid = B;
   p->grid = (int)(grid < 1 ? 1 : grid);

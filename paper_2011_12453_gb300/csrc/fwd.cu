@@ -172,7 +172,7 @@ struct FxPlan {
   FxArgs a;
   const void* kernel = nullptr;
   int grid = 0, warps = 0;
-  uint32_t smem = 0;
+  uint32_t smem = 0, smem_limit = 0;
   size_t ws_bytes = 0;
 };
 
@@ -205,6 +205,7 @@ gna_status fx_plan(const gna_graph* g, const Dims& m, int64_t B, FxPlan* p) {
   if (a.h_smem) a.oH = take(rows);
   if (o > budget) return GNA_ERR_UNSUPPORTED;
   p->smem = (uint32_t)o;
+  p->smem_limit = (uint32_t)budget;
   // tiles of 16 sites in equal rounds
   const int tiles = (N + 15) / 16, most = B <= di.sms ? 16 : 8, rounds = (tiles + most - 1) / most;
   p->warps = (tiles + rounds - 1) / rounds;
@@ -249,7 +250,7 @@ gna_status fx_run(const gna_graph* g, const Dims& m, const float* theta, const i
   p.a.B = B;
   p.a.logpsi = logpsi;
   p.a.gH = (float*)ws;
-  GNA_CUDA_TRY(cudaFuncSetAttribute(p.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem));
+  if ((st = allow_smem(p.kernel, p.smem_limit)) != GNA_OK) return st;
   void* args[] = {&p.a};
   GNA_CUDA_TRY(cudaLaunchKernel(p.kernel, dim3(p.grid), dim3(32 * p.warps), args, p.smem, stream));
   GNA_CUDA_TRY(cudaGetLastError());

@@ -946,7 +946,7 @@ static gna_status metro_plan(const gna_graph* g, const Dims& m, int64_t C, int w
   p->nwarps = nw;
   p->smem = (int)smem_for(nw);
   const void* kern = metro_kernel<T>(F, with_prop != 0);
-  GNA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
+  if ((st = allow_smem(kern, (uint64_t)di.smem_optin - 1024)) != GNA_OK) return st;
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 32 * nw, p->smem));
   if (occ > kMetroMaxWarps / nw) occ = kMetroMaxWarps / nw;

@@ -636,7 +636,7 @@ gna_status mt_plan(const gna_graph* g, const Dims& m, int64_t C, MtPlan* p) {
   warps = (int)((per_sm + rounds - 1) / rounds);
   a.warps = warps;
   p->smem = a.owarp + (uint32_t)warps * a.warp_bytes;
-  GNA_CUDA_TRY(cudaFuncSetAttribute(mt_kernel(m.F, form > 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p->smem));
+  if ((st = allow_smem(mt_kernel(m.F, form > 0), budget)) != GNA_OK) return st;
   const int64_t need = (C + warps - 1) / warps;
   p->grid = (int)(need < di.sms ? need : di.sms);
   // (the bytes of any number of chains up to C: fewer chains may be more warps)

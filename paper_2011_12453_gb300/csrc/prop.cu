@@ -481,7 +481,10 @@ static gna_status prop_run(bool grad, const gna_graph* g, const int8_t* spins, c
   *grid = prop_grid(B, g->d.E, &a.parts);
   const int smem = kSCfg * 4 + g->d.n * 8 + (g->d.n + 15) / 16 * 16;
   const void* k = grad ? (const void*)k_prop<true> : (const void*)k_prop<false>;
-  GNA_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  DeviceInfo di;
+  gna_status s = device_info(&di);
+  if (s == GNA_OK) s = allow_smem(k, (uint64_t)di.smem_optin - 64);
+  if (s != GNA_OK) return s;
   void* args[] = {&a};
   GNA_CUDA_TRY(cudaLaunchKernel(k, dim3(*grid), dim3(kPropThreads), args, smem, st));
   GNA_CUDA_TRY(cudaGetLastError());

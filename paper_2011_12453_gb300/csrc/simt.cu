@@ -1243,7 +1243,7 @@ gna_status simt_plan(const gna_graph* g, const Dims& m, int op, int64_t B, Plan*
     p->threads = kThreadsBwd / blocks;
   }
   const void* kp = kernel_ptr<T>(op);
-  GNA_CUDA_TRY(cudaFuncSetAttribute(kp, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem));
+  if ((st = allow_smem(kp, budget)) != GNA_OK) return st;
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kp, p->threads, p->smem));
   if (occ < 1) occ = 1;

@@ -1911,7 +1911,7 @@ static gna_status tc_plan(const gna_graph* g, const Dims& m, int op, int64_t B, 
   if (lay.smem_total < min_smem) lay.smem_total = min_smem;
   p->lay = lay;
   const void* kfn = split ? (const void*)k_tc<true> : (const void*)k_tc<false>;
-  GNA_CUDA_TRY(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lay.smem_total));
+  if ((st = allow_smem(kfn, budget)) != GNA_OK) return st;
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kfn, kTcThreads, lay.smem_total));
   if (occ < 1) occ = 1;
@@ -2050,7 +2050,7 @@ static gna_status tcb_plan(const gna_graph* g, const Dims& m, int64_t B, TcbPlan
   uint32_t smem = p->a.base.lay.smem_total;
   if (smem < min_smem) smem = min_smem;
   p->a.base.lay.smem_total = smem;
-  GNA_CUDA_TRY(cudaFuncSetAttribute((const void*)k_tc_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if ((st = allow_smem((const void*)k_tc_bwd, budget)) != GNA_OK) return st;
   int occ = 0;
   GNA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)k_tc_bwd, kTcThreads, smem));
   if (occ < 1) occ = 1;
