@@ -119,6 +119,18 @@ __device__ __forceinline__ double db_dtanh(double x, double2 hs, const double* p
   return d;
 }
 
+// The pair (H, S) of a move that is kept, back on S = 1 - H^2.  The factors of db_dtanh leave it by a
+// rounding, and the next ones enlarge what it is off: left alone it grew 1.5 times a sweep, until after some 100
+// sweeps H had no correct digit.  H decides below 0.75 and S above, where it has the digits; what is left is a
+// random walk of roundings, like that of Y (1e-14 after 10^4 moves).
+__device__ __forceinline__ double2 db_settle(double h, double s) {
+  if (fabs(h) < 0.75)
+    s = fma(-h, h, 1.0);
+  else
+    h = fma(0.5 * fma(-h, h, 1.0 - s), h, h);
+  return make_double2(h, s);
+}
+
 template <int FPL>
 __device__ void db_setup(const DbArgs& a, DbCtx& c) {
   const int F = a.m.F, N = a.m.N;
@@ -436,7 +448,7 @@ __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__
               const int r = i / F;
               const size_t o = (size_t)(l - 1) * NF + (size_t)(__ldg(rc + 2 * r) & 0xFFFF) * F + (i - r * F);
               Yc[o] = nw[3 * i];
-              Hc[o] = make_double2(nw[3 * i + 1], nw[3 * i + 2]);
+              Hc[o] = db_settle(nw[3 * i + 1], nw[3 * i + 2]);
             }
           }
           if (utid == 0) {
