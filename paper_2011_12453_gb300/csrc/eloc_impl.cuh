@@ -713,7 +713,8 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
   __syncthreads();
   for (int v = tid; v < N; v += kElThreads) {
     const int d = __ldg(a.g.row_ptr + v + 1) - __ldg(a.g.row_ptr + v);
-    ((float*)c.av)[v] = d > 0 ? (MODE == EL_X2 ? 1.f / sqrtf((float)d) : rsqrtf((float)d)) : 0.f;
+    // FP32: rounded once, as the forward's weights are; the BF16X2 operands (2^-16) do not see its last bit
+    ((float*)c.av)[v] = d > 0 ? (MODE == EL_X2 ? 1.f / sqrtf((float)d) : (float)(1.0 / sqrt((double)d))) : 0.f;
   }
   // Z^0 of a row that changes from up to down: (emb(-1) - emb(+1)) [W[:F] | W[F:]]
   for (int i = tid; i < 2 * F; i += kElThreads) {
