@@ -26,6 +26,8 @@
 // falls 3 to 5 times at weight scale 0.1.
 #pragma once
 
+#include <cfloat>
+
 #include "eloc.cuh"
 #include "frag.cuh"
 
@@ -892,7 +894,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
           float amp = expf(xr), sn, cs;
           sincosf(xi, &sn, &cs);
           if (MODE != EL_X2) {  // the parts of Delta below float32
-            amp = fmaf(amp, (float)(dre - (S)xr), amp);
+            if (amp <= FLT_MAX) amp = fmaf(amp, (float)(dre - (S)xr), amp);
             const float lo = (float)(dim - (S)xi), s0 = sn;
             sn = fmaf(cs, lo, sn);
             cs = fmaf(-s0, lo, cs);

@@ -146,3 +146,23 @@ def test_a_bias_that_is_not_a_number_shows_in_the_energy(torch, prec, name, scal
     s = torch.tensor(W.random_spins(g.n_sites, 8, seed=1), device="cuda")
     E = gna.local_energy(graph, model, theta, s, gna.ELOC_INCREMENTAL)
     assert torch.isnan(E[:, 0]).all()
+
+
+def test_a_ratio_beyond_float32_makes_the_energy_infinite(torch):
+    # real log Psi (Im w_r = 0) with ratios of up to exp(+-several hundred), summed with positive J
+    F, L = 16, 2
+    g = W.kagome(2)
+    th = W.random_theta(F, L, seed=1, scale=0.3)
+    o = 4 * F + 2 * F * F
+    th[o:o + 2 * F:2] *= 1000.0
+    th[o + 1:o + 2 * F:2] = 0.0
+    theta, th = _rounded(torch, th, F, "fp32")
+    graph, model = gna.Graph.from_workload(g, L), gna.Model(F, L, gna.PREC_FP32)
+    s = W.random_spins(g.n_sites, 40, seed=1)
+    st = torch.tensor(s, device="cuda")
+    Ah = gcn.norm_adjacency(gcn.adjacency(g.n_sites, g.edges))
+    d = np.nanmax(hz.bond_log_ratios(lambda x: gcn.logpsi_complex(th, F, L, Ah, x), g.edges, s).real, axis=1)
+    assert (d > 95).sum() > 10 and not ((d > 80) & (d < 95)).any()
+    for mode in (gna.ELOC_FULL, gna.ELOC_INCREMENTAL):
+        E = gna.local_energy(graph, model, theta, st, mode)[:, 0].cpu().numpy()
+        assert np.array_equal(np.isposinf(E), d > 95) and np.isfinite(E[d < 80]).all()
