@@ -61,11 +61,14 @@ typedef int32_t gna_status;
                                          (reported by gna_device_status) */
 
 /* Arithmetic of a call.  FP64: float64 everywhere (parity path).  FP32: float32
- * features, GEMMs and ratios.  BF16: the node-feature GEMM operands in bfloat16 on the
+ * features, GEMMs and ratios; the incremental local energy multiplies on the tensor cores,
+ * both operands as three bfloat16 terms (the six products above 2^-24), which keeps float32
+ * accuracy.  BF16: the node-feature GEMM operands in bfloat16 on the
  * tensor cores with float32 accumulation; everything else as FP32.  BF16X2: the same
  * tensor-core GEMMs with every float32 operand x carried as two bfloat16 values,
  * hi = bf16(x) and lo = bf16(x - hi) (about 16 significant bits), both multiplied and
- * accumulated in float32; feature rows in float32 and tanh to float32 accuracy.  W is a
+ * accumulated in float32 (three values, 24 bits, for the changes that the local energy
+ * propagates); feature rows in float32 and tanh to float32 accuracy.  W is a
  * bfloat16 model parameter in both tensor-core modes (the float32 theta is rounded).  The
  * backward (gna_backward) always splits its operands; the sampler runs BF16 for both.
  * Reductions across samples (energies, weights, gradients) are float64 in every mode. */

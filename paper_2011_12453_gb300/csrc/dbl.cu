@@ -8,10 +8,12 @@
 //   - the rows of ball_{l-1} are multiplied instead of those of ball_l (Kagome 2x2x3, L 2: 7 rows
 //     a bond instead of 19);
 //   - tanh(Y + x) - tanh(Y) comes from a rational tanh(x) and the cached H = tanh Y and 1 - H^2 with
-//     one reciprocal (13 instructions an element, 20 with the updates of H and 1 - H^2 that an
-//     accepted move copies; exp, tanh and a division took 70);
+//     one reciprocal (13 instructions an element, 20 with the updates of H and 1 - H^2 and 5 more when an
+//     accepted move keeps them; exp, tanh and a division took 70);
 //   - a warp holds 32 / F rows of F <= 16 features, not one;
 //   - blocks of four warps, so that 1024 chains reach every SM (16 chains a block filled 64 SMs).
+// Ten sweeps of 1024 chains, Kagome 2x2x3, L 2, F 16: 23.9 -> 3.01 ms (the general kernels before, these
+// after); update of 1024 configurations 1.00 -> 0.88.
 #include <climits>
 #include <cmath>
 #include <cstring>

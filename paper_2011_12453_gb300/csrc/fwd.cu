@@ -11,7 +11,8 @@
 // a configuration has tiles (at most 8, so that several blocks share an SM; 16 while every block has
 // an SM to itself), no warp waits for another's second tile.
 // Triangular 144, L 4, F 48: 1000 configurations 87 us against some 270, 4001 configurations and
-// their gradient 4.29 -> 3.59 ms; one configuration of Kagome 108, L 4, F 32, through the library 37 -> 33 us.
+// their gradient 4.29 -> 3.59 ms.  One configuration through the library is bound by the host's call:
+// Kagome 108, L 4, F 32 takes 34 to 37 us with either kernel.
 #include <cstring>
 
 #include "eloc_impl.cuh"

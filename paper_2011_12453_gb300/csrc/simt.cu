@@ -979,9 +979,10 @@ __global__ void __launch_bounds__(kThreads) k_metropolis(const SimtArgs<T> a) {
 // SM (128 registers each), as four blocks of 128, two of 256 or one of 512 threads.  The phases of
 // a small sample occupy few threads (2F F / 4 of them in dW), and other samples' blocks fill in:
 // update of 1024 configurations, F 16, FP64 Kagome 2x2x3 0.81 -> 0.71 ms with four blocks, FP32 bosons on
-// 108 sites 1.28 -> 1.13.  One block where F F / 2 threads find work in it, where the features are in
-// the workspace (a drawn FP32 gradient took 12 % longer with four), and where the last round of
-// samples would leave more of the smaller blocks idle than they gain (a fifth).
+// 108 sites 1.28 -> 1.13.  One block where F F / 2 threads find work in it, where the features are in the
+// workspace (1216 gradients, F 16: FP32 on Kagome 432, L 6, 2.64 ms with one and 2.90 with four; FP64 on 300
+// sites, L 4, has it the other way, 6.00 against 5.33), and where the last round of samples would leave more
+// of the smaller blocks idle than they gain (a fifth).
 constexpr int kThreadsBwd = 512;
 
 template <typename T>

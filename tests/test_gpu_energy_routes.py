@@ -67,6 +67,7 @@ def test_shallow_split_operand_model_on_many_sites(torch, n, F):
     st = torch.tensor(s, device="cuda")
     gna.device_status(clear=True)
     E, dl = gna.local_energy(graph, model, theta, st, gna.ELOC_INCREMENTAL, bonds=True)
+    assert torch.equal(gna.local_energy_logpsi(graph, model, theta, st)[1], gna.forward(graph, model, theta, st))
     assert gna.device_status(clear=True) == 0
     delta, bd, eb = BD.bond_bounds(th, F, L, Ah, g.edges, g.J, s, "bf16x2")
     anti = ~np.isnan(delta.real)
