@@ -304,6 +304,32 @@ def run_reference(a):
 # our arm
 # ---------------------------------------------------------------------------------
 
+# DRAM bytes per sample of the dominant kernels from one ncu capture (dram__bytes_read.sum +
+# dram__bytes_write.sum of one launch of 2048 configurations or chains), valid only for the
+# source files that were profiled (SHA-256 of their concatenation).
+PROFILED_TRAFFIC = {
+    ("kagome_6x6x3_heisenberg", "k_eloc"): ((2641408 + 743424) / 2048, ("eloc.cu", "eloc_impl.cuh", "frag.cuh"),
+                                            "cebed13631ea8b0a720dfe6912961deb9ca9b89960f5dbc7bb77c7dcf08ae639"),
+    ("kagome_6x6x3_heisenberg", "k_tc<0>"): ((3075072 + 861440) / 2048, ("tc.cu", "frag.cuh"),
+                                             "e4e674babb2bf87ca0786d9538540d126dd4b57595daa8c24303a657a468ce91"),
+    ("kagome_6x6x3_heisenberg", "k_mt_metro"): ((7909376 + 123260672) / 2048, ("mtile.cu", "frag.cuh"),
+                                                "0b25548d5e2dec1b62fff6f06ff3fe760e5b2d4b6b026cd8d584d72df1d18955"),
+}
+
+
+def profiled_traffic(workload, kernel, units):
+    import hashlib
+
+    rec = PROFILED_TRAFFIC.get((workload, kernel))
+    if rec is None:
+        return None
+    h = hashlib.sha256()
+    for name in rec[1]:
+        with open(os.path.join(ROOT, "paper_2011_12453_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return rec[0] * units if h.hexdigest() == rec[2] else None
+
+
 def sweep_flops(g, F, L, ball, deg_of, spins_np, steps_per_chain):
     """Expected algorithmic FLOPs of `steps_per_chain` plain exchange proposals per chain: the
     bond is uniform over the edges, an antiparallel bond costs
@@ -328,7 +354,7 @@ def measure_workload(key, prec_name, dev, flush, K_timed, peaks, peak_kind):
     min(K, K_timed) reuse updates over all S x C samples (incremental local energy with log Psi,
     ISGO weights, backward + SGD; L2 flushed before each).  Reports the mean update (the ISGO
     step), the iteration (sweeps + K updates; extrapolated from the timed updates when
-    K_timed < K), local-energy samples/s with the roofline of k_tc, and the energy agreement
+    K_timed < K), local-energy samples/s with the roofline of that kernel, and the energy agreement
     with the plain FP32 full re-evaluation on a subset of the samples."""
     import torch
 
@@ -577,7 +603,7 @@ def run_ours(a):
                     "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                     "kernel": "k_mt_metro (gna_metropolis_sweep, %d sweeps, BF16 mma.sync)" % S,
                     "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl_sweep,
-                    "traffic": None}
+                    "traffic": profiled_traffic(wl["workload"], "k_mt_metro", C * S)}
         else:
             roof = {"bound": "alu", "achieved": fl_sweep / (t_sweep / 1000.0) / 1e12, "peak": alu_peak,
                     "unit": "TFLOP/s", "kernel": "k_metro_warp (gna_metropolis_sweep, %d sweeps)" % S,
@@ -589,7 +615,7 @@ def run_ours(a):
                 "kernel": ("k_eloc (gna_local_energy_logpsi, split BF16 operands, mma.sync)"
                            if prec == gna.PREC_BF16X2 else "k_tc<0> (gna_local_energy_logpsi, BF16 tcgen05)"),
                 "peak_source": peak_kind + " bf16_tflops_sustained", "flops_per_launch": fl_incr,
-                "traffic": None}
+                "traffic": profiled_traffic(wl["workload"], "k_eloc" if prec == gna.PREC_BF16X2 else "k_tc<0>", Bn)}
     else:
         roof = {"bound": "alu", "achieved": fl_incr / (t_incr / 1000.0) / 1e12, "peak": alu_peak,
                 "unit": "TFLOP/s", "kernel": "k_eloc (gna_local_energy incremental, FP32)",
@@ -648,7 +674,7 @@ def run_ours(a):
             "e2e": {"value": e2e_value, "unit": "samples/s", "h2d_bytes_per_step": int(C * N),
                     "d2h_bytes_per_step": 32},
             # per step: the sweep, then per update the local energy with log Psi (one launch on the
-            # tensor cores, forward + local energy otherwise), 4 weight kernels, backward + its
+            # tensor cores, forward + local energy otherwise), 2 weight kernels, backward + its
             # reduction, SGD
             "gpu_launches": int(Ksteps * (1 + (6 if prec in (gna.PREC_BF16, gna.PREC_BF16X2) else 7) * K)),
             "clocks": clk,
