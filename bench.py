@@ -309,11 +309,11 @@ def run_reference(a):
 # source files that were profiled (SHA-256 of their concatenation).
 PROFILED_TRAFFIC = {
     ("kagome_6x6x3_heisenberg", "k_eloc"): ((2641408 + 743424) / 2048, ("eloc.cu", "eloc_impl.cuh", "frag.cuh"),
-                                            "cebed13631ea8b0a720dfe6912961deb9ca9b89960f5dbc7bb77c7dcf08ae639"),
+                                            "dec715d3b06dabeb18c50297aece4485f883b90104bdffea1875ea633189c538"),
     ("kagome_6x6x3_heisenberg", "k_tc<0>"): ((3075072 + 861440) / 2048, ("tc.cu", "frag.cuh"),
-                                             "e4e674babb2bf87ca0786d9538540d126dd4b57595daa8c24303a657a468ce91"),
+                                             "e1280f51ad0e791b3ba2f8769a90c18c1ab1fc36e446467898fab93a9f6be721"),
     ("kagome_6x6x3_heisenberg", "k_mt_metro"): ((7909376 + 123260672) / 2048, ("mtile.cu", "frag.cuh"),
-                                                "0b25548d5e2dec1b62fff6f06ff3fe760e5b2d4b6b026cd8d584d72df1d18955"),
+                                                "39dc170ec26274c533d391fec4f5829d4a27230a5b4a795e0730b75f7a542430"),
 }
 
 

@@ -123,8 +123,8 @@ __device__ __forceinline__ double db_dtanh(double x, double2 hs, const double* p
 
 // The pair (H, S) of a move that is kept, back on S = 1 - H^2.  The factors of db_dtanh leave it by a
 // rounding, and the next ones enlarge what it is off: left alone it grew 1.5 times a sweep, until after some
-// 100 sweeps (Kagome 2x2x3, weight scale 0.3) H had no correct digit.  H decides below 0.75 and S above, where it has the digits; what is left is a
-// random walk of roundings, like that of Y (1e-14 after 10^4 moves).
+// 100 sweeps (Kagome 2x2x3, weight scale 0.3) H had no correct digit.  H decides below 0.75 and S above,
+// where it has the digits; what is left is a random walk of roundings, like that of Y (1e-14 after 10^4 moves).
 __device__ __forceinline__ double2 db_settle(double h, double s) {
   if (fabs(h) < 0.75)
     s = fma(-h, h, 1.0);
@@ -133,7 +133,9 @@ __device__ __forceinline__ double2 db_settle(double h, double s) {
   return make_double2(h, s);
 }
 
-template <int FPL>
+// FINITE_W: an infinite weight becomes one that saturates tanh as well, so that a unit whose input does not change
+// stays out of the energy (0 w = 0), as where the rows are recomputed.
+template <bool FINITE_W>
 __device__ void db_setup(const DbArgs& a, DbCtx& c) {
   const int F = a.m.F, N = a.m.N;
   const double* th = a.theta;
@@ -144,7 +146,10 @@ __device__ void db_setup(const DbArgs& a, DbCtx& c) {
   double* br = (double*)(db_smem + a.obr);
   double* av = (double*)(db_smem + a.oav);
   double* z0 = (double*)(db_smem + a.oz0);
-  for (int i = threadIdx.x; i < 2 * F * F; i += blockDim.x) W[i] = th[a.m.oW + i];
+  for (int i = threadIdx.x; i < 2 * F * F; i += blockDim.x) {
+    const double w = th[a.m.oW + i];
+    W[i] = FINITE_W && fabs(w) == INFINITY ? copysign(1e200, w) : w;
+  }
   for (int i = threadIdx.x; i < F; i += blockDim.x) b[i] = th[a.m.ob + i];
   for (int i = threadIdx.x; i < 2 * F; i += blockDim.x) emb[i] = tanh(th[a.m.oWe + i] + th[a.m.obe + i % F]);
   for (int i = threadIdx.x; i < (F + 2) * 2; i += blockDim.x) wr[i] = th[a.m.owr + i];
@@ -359,7 +364,7 @@ __device__ __forceinline__ void db_delta(const DbCtx& c, int info, const int8_t*
 template <int FPL>
 __global__ void __launch_bounds__(kDbThreads) k_db_metro(const __grid_constant__ DbArgs a) {
   DbCtx c;
-  db_setup<FPL>(a, c);
+  db_setup<false>(a, c);
   const int N = a.m.N, F = a.m.F, L = a.m.L, E = a.m.E, lane = c.lane;
   const int warp = threadIdx.x >> 5, h = warp / a.uw, uwarp = warp % a.uw, uthreads = a.uw * 32, utid = threadIdx.x - h * uthreads;
   if (h >= a.units) return;
@@ -516,7 +521,7 @@ __global__ void __launch_bounds__(kDbThreads) k_db_eloc(const __grid_constant__ 
   __shared__ int s_cnt[kDbWarps];
   __shared__ double s_e[3 * kDbWarps];
   DbCtx c;
-  db_setup<FPL>(a, c);
+  db_setup<true>(a, c);
   const int N = a.m.N, F = a.m.F, L = a.m.L, E = a.m.E, lane = c.lane;
   const int warp = threadIdx.x >> 5, h = warp / a.uw, uwarp = warp % a.uw, uthreads = a.uw * 32;
   const bool active = h < a.units;

@@ -690,7 +690,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
   const float* W = th + a.m.oW;
   // parameters and graph: once per CTA
   for (int i = tid; i < el_wterms(MODE) * 2 * FC * FC * 32; i += kElThreads)
-    ((uint4*)c.Wf)[i] = make_wfrag<FC>(W, (i / (FC * 32)) % (2 * FC), (i / 32) % FC, i & 31, i / (2 * FC * FC * 32));
+    ((uint4*)c.Wf)[i] = make_wfrag<FC, MODE == EL_F32>(W, (i / (FC * 32)) % (2 * FC), (i / 32) % FC, i & 31, i / (2 * FC * FC * 32));
   for (int i = tid; i < F; i += kElThreads) ((float*)c.bias)[i] = th[a.m.ob + i];
   if (MODE != EL_F32_LN) {
     for (int i = tid; i < 2 * F; i += kElThreads) ((float*)c.emb)[i] = tanhf(th[a.m.oWe + i] + th[a.m.obe + i % F]);
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(kElThreads, 1) k_eloc(const __grid_constant__ 
     const int f = i % F, top = i < F ? 0 : F;
     float z = 0.f;
     for (int k = 0; k < F; ++k) {
-      const float w = W[(size_t)(top + k) * F + f];
+      const float w = MODE == EL_F32 ? finite_w(W[(size_t)(top + k) * F + f]) : W[(size_t)(top + k) * F + f];
       z = fmaf(c.emb[F + k] - c.emb[k], MODE == EL_X2 ? __bfloat162float(__float2bfloat16_rn(w)) : w, z);
     }
     ((float*)c.z0)[i] = z;

@@ -85,11 +85,14 @@ __device__ __forceinline__ void split3(uint64_t m1, float a, float b, uint32_t& 
 // ((kc * FC + c) * 32 + lane) holds, for K step kc (16 rows of W) and output chunk c, the
 // registers (b0, b1) of column tile 2c and (b0, b1) of column tile 2c + 1.
 // term: 0 = bf16(w), 1 = bf16 of what that leaves, 2 = bf16 of what both leave.
+// (an infinite w of a split in terms becomes one that saturates tanh as well, so that the terms stay numbers)
+constexpr float kSaturatingW = 1e30f;
+__device__ __forceinline__ float finite_w(float w) { return fabsf(w) == INFINITY ? copysignf(kSaturatingW, w) : w; }
 __device__ __forceinline__ float wterm(float w, int term) {
   for (int t = 0; t < term; ++t) w -= __bfloat162float(__float2bfloat16_rn(w));
   return w;
 }
-template <int FC>
+template <int FC, bool TERMS = false>
 __device__ __forceinline__ uint4 make_wfrag(const float* W, int kc, int c, int lane, int term) {
   constexpr int F = 16 * FC;
   const int n = lane >> 2, q = lane & 3;
@@ -97,8 +100,12 @@ __device__ __forceinline__ uint4 make_wfrag(const float* W, int kc, int c, int l
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float* w = W + (size_t)(16 * kc + 4 * q) * F + 16 * c + 4 * (n >> 1) + 2 * h + (n & 1);
-    const __nv_bfloat162 x = __floats2bfloat162_rn(wterm(w[0], term), wterm(w[F], term));
-    const __nv_bfloat162 y = __floats2bfloat162_rn(wterm(w[2 * F], term), wterm(w[3 * F], term));
+    float t[4] = {w[0], w[F], w[2 * F], w[3 * F]};
+    if (TERMS)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) t[i] = finite_w(t[i]);
+    const __nv_bfloat162 x = __floats2bfloat162_rn(wterm(t[0], term), wterm(t[1], term));
+    const __nv_bfloat162 y = __floats2bfloat162_rn(wterm(t[2], term), wterm(t[3], term));
     r[2 * h] = *reinterpret_cast<const uint32_t*>(&x);
     r[2 * h + 1] = *reinterpret_cast<const uint32_t*>(&y);
   }

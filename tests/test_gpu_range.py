@@ -166,3 +166,22 @@ def test_a_ratio_beyond_float32_makes_the_energy_infinite(torch):
     for mode in (gna.ELOC_FULL, gna.ELOC_INCREMENTAL):
         E = gna.local_energy(graph, model, theta, st, mode)[:, 0].cpu().numpy()
         assert np.array_equal(np.isposinf(E), d > 95) and np.isfinite(E[d < 80]).all()
+
+
+@pytest.mark.parametrize("prec,tol", [("fp32", 1e-5), ("fp64", 1e-9)])
+@pytest.mark.parametrize("F,L,sign", [(16, 1, 1.0), (32, 3, -1.0)])
+def test_an_infinite_weight_saturates_its_unit(torch, prec, tol, F, L, sign):
+    # as in the recomputing mode: tanh(+-inf) = +-1, and where the unit's input does not change its 0 x inf is no term
+    g = W.kagome(3)
+    theta, th = _rounded(torch, W.random_theta(F, L, seed=F, scale=0.3), F, prec)
+    theta[3 * F + 7] = sign * float("inf")
+    th[3 * F + 7] = sign * 1e30
+    graph, model = gna.Graph.from_workload(g, L), gna.Model(F, L, PREC[prec])
+    s = W.random_spins(g.n_sites, 5, seed=3)
+    st = torch.tensor(s, device="cuda")
+    full = gna.local_energy(graph, model, theta, st, gna.ELOC_FULL)
+    E = gna.local_energy(graph, model, theta, st, gna.ELOC_INCREMENTAL)
+    assert torch.isfinite(full).all()
+    Ah = gcn.norm_adjacency(gcn.adjacency(g.n_sites, g.edges))
+    lim = 2 * tol * np.maximum(SC.eloc_scale(th, F, L, Ah, g.edges, g.J, s), 1.0)
+    assert np.all((E - full).abs().cpu().numpy().max(axis=1) <= lim)
